@@ -167,43 +167,11 @@ constexpr float kDegenerateGap = 2e-2f;
 // re-solve there would not change the result's accuracy, only its cost (FP64
 // runs at a small fraction of the FP32 rate).
 constexpr float kDegenerateGapMixed = 1e-2f;
-// The same for the FP64 closed form (the mixed form's re-solve).  Near a double
-// root an error eps in det(B) / 2 moves l1 by about eps p^2 / gap and the null
-// vector by that over the gap, eps (p / gap)^2: at a gap of 1e-4 of the spread
-// and eps = 1.1e-16 that is ~1e-8, far below the FP32 outputs' resolution,
-// so only voxels closer than that go on to FP64 Jacobi.
-constexpr double kDegenerateGap64 = 1e-4;
 
 template <typename T>
 struct Sym3 {
   T a, b, c, d, e, f;  // xx, yy, zz, xy, xz, yz
 };
-
-// Eigenvector of eigenvalue lam: the largest of the three cross products of
-// the rows of (S - lam I).  Returns the squared norm of the chosen product
-// before normalisation (0 when S - lam I has rank <= 1).
-template <typename T>
-__device__ __forceinline__ T null_vector(const Sym3<T>& s, T lam, T v[3]) {
-  T r0x = s.a - lam, r0y = s.d, r0z = s.e;
-  T r1x = s.d, r1y = s.b - lam, r1z = s.f;
-  T r2x = s.e, r2y = s.f, r2z = s.c - lam;
-  T x01 = r0y * r1z - r0z * r1y, y01 = r0z * r1x - r0x * r1z, z01 = r0x * r1y - r0y * r1x;
-  T x02 = r0y * r2z - r0z * r2y, y02 = r0z * r2x - r0x * r2z, z02 = r0x * r2y - r0y * r2x;
-  T x12 = r1y * r2z - r1z * r2y, y12 = r1z * r2x - r1x * r2z, z12 = r1x * r2y - r1y * r2x;
-  T n01 = x01 * x01 + y01 * y01 + z01 * z01;
-  T n02 = x02 * x02 + y02 * y02 + z02 * z02;
-  T n12 = x12 * x12 + y12 * y12 + z12 * z12;
-  T bx = x01, by = y01, bz = z01, bn = n01;
-  if (n02 > bn) { bx = x02; by = y02; bz = z02; bn = n02; }
-  if (n12 > bn) { bx = x12; by = y12; bz = z12; bn = n12; }
-  if (bn > T(0)) {
-    T inv = T(1) / sqrt(bn);
-    v[0] = bx * inv; v[1] = by * inv; v[2] = bz * inv;
-  } else {
-    v[0] = T(1); v[1] = T(0); v[2] = T(0);
-  }
-  return bn;
-}
 
 // Closed-form eigenvalues (trigonometric solution of the characteristic cubic,
 // O. K. Smith, Comm. ACM 4(4), 1961) and the smallest-eigenvalue eigenvector.
@@ -216,11 +184,7 @@ __device__ __forceinline__ T null_vector(const Sym3<T>& s, T lam, T v[3]) {
 // reciprocal square roots from rsqrt; the errors they add, a few 1e-7 of p,
 // are far below what the re-solve threshold leaves between l1 and l2.
 // The FP32 form lists the voxel for a re-solve when l2 - l1 < gap (l3 - l1).
-template <typename T>
-__device__ __forceinline__ bool eig_closed(const Sym3<T>& s, T l[3], T v[3], T gap);
-
-template <>
-__device__ __forceinline__ bool eig_closed<float>(const Sym3<float>& s, float l[3], float v[3], float gap) {
+__device__ __forceinline__ bool eig_closed(const Sym3<float>& s, float l[3], float v[3], float gap) {
   const float q = (s.a + s.b + s.c) * (1.f / 3.f);
   const float aq = s.a - q, bq = s.b - q, cq = s.c - q;
   const float p1 = s.d * s.d + s.e * s.e + s.f * s.f;
@@ -267,35 +231,99 @@ __device__ __forceinline__ bool eig_closed<float>(const Sym3<float>& s, float l[
   return (l2 - l1) >= gap * (l3 - l1) && bn > 0.f;
 }
 
-// FP64 version (the re-solve of the mixed form): library acos / sincos / sqrt,
-// l1 from the same sin and cos as l3 (one sincos instead of two cos).
-template <>
-__device__ __forceinline__ bool eig_closed<double>(const Sym3<double>& s, double l[3], double v[3], double gap) {
-  const double q = (s.a + s.b + s.c) / 3.0;
-  const double aq = s.a - q, bq = s.b - q, cq = s.c - q;
-  const double p1 = s.d * s.d + s.e * s.e + s.f * s.f;
-  const double p2 = aq * aq + bq * bq + cq * cq + 2.0 * p1;
-  if (p2 == 0.0) {
-    l[0] = l[1] = l[2] = q;
-    v[0] = 1.0; v[1] = 0.0; v[2] = 0.0;
-    return true;
+// Newton's iteration for 1 / sqrt(x) and 1 / x in FP64 from FP32 starts: two
+// steps take their 1e-7 to FP64 rounding.
+__device__ __forceinline__ double rsqrt_newton(double x) {
+  double y = (double)rsqrtf((float)x);
+#pragma unroll
+  for (int k = 0; k < 2; ++k) y = fma(0.5 * y, fma(-(x * y), y, 1.0), y);
+  return y;
+}
+__device__ __forceinline__ double rcp_newton(double x) {
+  double y = (double)__frcp_rn((float)x);
+#pragma unroll
+  for (int k = 0; k < 2; ++k) y = fma(y, fma(-x, y, 1.0), y);
+  return y;
+}
+
+// The FP64 re-solve of the mixed form, by deflation: the eigenvalue that lies
+// apart from the other two (of B = S - qI, the extreme root on the side of the
+// sign of det B) by Newton's iteration on the characteristic cubic
+// mu^3 - 3 p^2 mu - det B from its FP32 trigonometric value, its eigenvector w
+// from the adjugate of B - mu I, and, where that is the largest one, the two
+// smallest from the 2 x 2 problem of B in the plane across w (an orthonormal
+// basis of it as in Duff et al., J. Computer Graphics Techniques 6(1), 2017).
+// Deflating first leaves an error of eps p / gap in the direction, where a
+// closed form for all three roots has eps (p / gap)^2 and needs a fallback
+// near a double root.  About 130 FP64 operations without library calls: FP64
+// runs at 2 lanes per clock and SM here, so their number is the re-solve's
+// time: 243 000 tensors 302 us with acos, sincos and a Jacobi fallback below
+// a gap of 1e-4, 89 us now (the FP64 pipe 78% busy).
+// False (nothing written) where p is below 1e-3 of the largest entry or the
+// pair lies within 1e-10 p: the caller's Jacobi then takes the voxel.
+__device__ __forceinline__ bool eig_deflate(const Sym3<float>& s, float l[3], float v[3]) {
+  // scaled by a power of two to entries of at most 2 (exact)
+  const float big = fmaxf(fmaxf(fmaxf(fabsf(s.a), fabsf(s.b)), fmaxf(fabsf(s.c), fabsf(s.d))),
+                          fmaxf(fabsf(s.e), fabsf(s.f)));
+  if (!(big > 1e-37f && big < 1e37f)) return false;
+  const int ex = (__float_as_int(big) >> 23) - 127;
+  const float down = __int_as_float((127 - ex) << 23), up = __int_as_float((127 + ex) << 23);
+  const double sa = (double)(s.a * down), sb = (double)(s.b * down), sc = (double)(s.c * down);
+  const double d = (double)(s.d * down), e = (double)(s.e * down), f = (double)(s.f * down);
+  const double q = (sa + sb + sc) * (1.0 / 3.0);
+  const double a = sa - q, b = sb - q, c = sc - q;
+  const double P = (0.5 * fma(a, a, fma(b, b, c * c)) + fma(d, d, fma(e, e, f * f))) * (1.0 / 3.0);  // p^2
+  const double det = fma(a, fma(b, c, -(f * f)), fma(d, fma(e, f, -(d * c)), e * fma(d, f, -(b * e))));
+  const float Pf = (float)P;
+  if (!(Pf > 1e-6f)) return false;
+  const float ip = rsqrtf(Pf), rf = 0.5f * (float)det * ip * ip * ip;
+  const bool top = rf >= 0.f;
+  const float mu0 = copysignf(2.f * Pf * ip * __cosf(acosf(fminf(fabsf(rf), 1.f)) * (1.f / 3.f)), rf);
+  const double inv_slope = (double)__fdividef(1.f, 3.f * (mu0 * mu0 - Pf));  // mu0^2 >= 3 p^2
+  double mu = (double)mu0;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) mu = fma(-fma(mu, fma(mu, mu, -3.0 * P), -det), inv_slope, mu);
+  // w: the adjugate's column with the largest diagonal entry
+  const double A = a - mu, B = b - mu, C = c - mu;
+  const double c00 = fma(B, C, -(f * f)), c11 = fma(A, C, -(e * e)), c22 = fma(A, B, -(d * d));
+  const double c01 = fma(e, f, -(d * C)), c02 = fma(d, f, -(B * e)), c12 = fma(d, e, -(A * f));
+  double x = c00, y = c01, z = c02;
+  if (c11 > c00 && c11 >= c22) { x = c01; y = c11; z = c12; }
+  if (c22 > c00 && c22 > c11) { x = c02; y = c12; z = c22; }
+  double m1, m2;  // the other two eigenvalues of B, ascending
+  if (top) {
+    const double iw = rsqrt_newton(fma(x, x, fma(y, y, z * z)));
+    x *= iw; y *= iw; z *= iw;
+    const double sg = z >= 0.0 ? 1.0 : -1.0, g = -rcp_newton(sg + z), h = x * y * g;
+    const double u0 = fma(sg * x, x * g, 1.0), u1 = sg * h, u2 = -sg * x;
+    const double w0 = h, w1 = fma(y * y, g, sg), w2 = -y;
+    const double t0 = fma(a, u0, fma(d, u1, e * u2)), t1 = fma(d, u0, fma(b, u1, f * u2)),
+                 t2 = fma(e, u0, fma(f, u1, c * u2));
+    // half the difference of the 2 x 2 diagonal (its sum is -mu) and the off-diagonal entry
+    const double t = fma(u0, t0, fma(u1, t1, fma(u2, t2, 0.5 * mu)));
+    const double o = fma(w0, t0, fma(w1, t1, w2 * t2));
+    const double hh = fma(t, t, o * o);
+    if (!(hh > 1e-20 * P)) return false;
+    const double r = hh * rsqrt_newton(hh);
+    const double k0 = t >= 0.0 ? -o : r - t, k1 = t >= 0.0 ? t + r : -o;
+    x = fma(k0, u0, k1 * w0);
+    y = fma(k0, u1, k1 * w1);
+    z = fma(k0, u2, k1 * w2);
+    m1 = fma(-0.5, mu, -r);
+    m2 = fma(-0.5, mu, r);
+    l[0] = (float)(q + m1) * up;
+    l[1] = (float)(q + m2) * up;
+    l[2] = (float)(q + mu) * up;
+  } else {  // the smallest one lies apart: w is its vector
+    const double r = sqrt(fmax(3.0 * fma(-0.25 * mu, mu, P), 0.0));
+    m1 = fma(-0.5, mu, -r);
+    m2 = fma(-0.5, mu, r);
+    l[0] = (float)(q + mu) * up;
+    l[1] = (float)(q + m1) * up;
+    l[2] = (float)(q + m2) * up;
   }
-  const double p = sqrt(p2 / 6.0);
-  const double ip = 1.0 / p;
-  const double B00 = aq * ip, B11 = bq * ip, B22 = cq * ip, B01 = s.d * ip, B02 = s.e * ip, B12 = s.f * ip;
-  const double det = B00 * (B11 * B22 - B12 * B12) - B01 * (B01 * B22 - B12 * B02) + B02 * (B01 * B12 - B11 * B02);
-  const double r = fmin(fmax(0.5 * det, -1.0), 1.0);
-  const double phi = acos(r) / 3.0;
-  double sp, cp;
-  sincos(phi, &sp, &cp);
-  double l3 = q + 2.0 * p * cp;
-  double l1 = q - p * (cp + 1.7320508075688772935 * sp);
-  double l2 = 3.0 * q - l1 - l3;
-  if (l2 < l1) { double t = l1; l1 = l2; l2 = t; }
-  if (l3 < l2) { double t = l2; l2 = l3; l3 = t; }
-  l[0] = l1; l[1] = l2; l[2] = l3;
-  const double bn = null_vector(s, l1, v);
-  return (l2 - l1) >= gap * (l3 - l1) && bn > 0.0;
+  v[0] = (float)x; v[1] = (float)y; v[2] = (float)z;
+  return true;
 }
 
 // Cyclic Jacobi (Golub & Van Loan, Matrix Computations, section 8.5) on a

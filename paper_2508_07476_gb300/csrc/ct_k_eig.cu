@@ -7,8 +7,8 @@
 // characteristic cubic, cross product of two rows of S - l1 I).  Voxels whose
 // two smallest eigenvalues nearly coincide, where that form loses half of its
 // digits, are appended to a compact list and re-solved by a second kernel:
-// FP32 cyclic Jacobi in the FP32 form, FP64 closed form (FP64 Jacobi if that
-// too is near-degenerate) in the mixed form.  The list keeps the re-solve off
+// FP32 cyclic Jacobi in the FP32 form, FP64 deflation (FP64 Jacobi where even
+// that has no gap to work with) in the mixed form.  The list keeps the re-solve off
 // the common path, so no warp diverges into it.
 #include <algorithm>
 
@@ -32,12 +32,14 @@ __device__ __forceinline__ Sym3<float> load_sym(const float* S, int64_t n, int64
 // Robust re-solve of one voxel.
 __device__ __forceinline__ void resolve(const Sym3<float>& s, bool mixed, float l[3], float v[3]) {
   if (mixed) {
-    Sym3<double> sd{(double)s.a, (double)s.b, (double)s.c, (double)s.d, (double)s.e, (double)s.f};
-    double ld[3], vd[3];
-    if (!eig_closed<double>(sd, ld, vd, kDegenerateGap64)) eig_jacobi<double>(sd, ld, vd);
-    for (int k = 0; k < 3; ++k) {
-      l[k] = (float)ld[k];
-      v[k] = (float)vd[k];
+    if (!eig_deflate(s, l, v)) {
+      Sym3<double> sd{(double)s.a, (double)s.b, (double)s.c, (double)s.d, (double)s.e, (double)s.f};
+      double ld[3], vd[3];
+      eig_jacobi<double>(sd, ld, vd);
+      for (int k = 0; k < 3; ++k) {
+        l[k] = (float)ld[k];
+        v[k] = (float)vd[k];
+      }
     }
   } else {
     eig_jacobi<float>(s, l, v);
@@ -104,7 +106,7 @@ __global__ void __launch_bounds__(256, CT_EIG_MINB)
   float l[3] = {0.f, 0.f, 0.f}, v[3] = {1.f, 0.f, 0.f};
   if (inside) {
     const Sym3<float> s = load_sym(S, box_vox(sb), box_index(sb, x, y, z));
-    if (!eig_closed<float>(s, l, v, fb.gap)) push_fallback(fb, ((int64_t)zr * ob.n[1] + yr) * ob.n[0] + (x - ob.lo[0]));
+    if (!eig_closed(s, l, v, fb.gap)) push_fallback(fb, ((int64_t)zr * ob.n[1] + yr) * ob.n[0] + (x - ob.lo[0]));
   }
   write_voxel<VT, AT, FT>(o, box_index(o.ab, x, y, z), inside, F, x, y, z, l, v, fill);
 }
@@ -134,7 +136,7 @@ __device__ __forceinline__ void eig32_body(const float* __restrict__ S, Box sb, 
     s.d = __ldg(S + 3 * ns + si);
     s.e = __ldg(S + 4 * ns + si);
     s.f = __ldg(S + 5 * ns + si);
-    if (!eig_closed<float>(s, l, v, fb.gap))
+    if (!eig_closed(s, l, v, fb.gap))
       push_fallback(fb, ((int64_t)blk.z() * ob.n[1] + blk.y()) * ob.n[0] + (x - ob.lo[0]));
   }
   write_voxel<VT, AT, FT, int, PLAIN>(o, box_index32(o.ab, x, y, z), inside, F, x, y, z, l, v, fill);
@@ -239,7 +241,7 @@ __device__ __forceinline__ void eig_compact_body(const float* __restrict__ S, Bo
       if (i0 + kEigThreads * u >= total) break;
       const int x = xs[u];
       float l[3], v[3];
-      if (!eig_closed<float>(s[u], l, v, fb.gap))
+      if (!eig_closed(s[u], l, v, fb.gap))
         push_fallback(fb, ((int64_t)blk.z() * ob.n[1] + blk.y()) * ob.n[0] + (x - ob.lo[0]));
       write_voxel<VT, AT, FT, int, PLAIN>(o, box_index32(o.ab, x, y, z), true, F, x, y, z, l, v, fill);
     }
@@ -456,7 +458,7 @@ __global__ void __launch_bounds__(256)
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     Sym3<float> s = load_sym(S, n, i);
     float l[3], v[3];
-    if (!eig_closed<float>(s, l, v, fb.gap)) push_fallback(fb, i);
+    if (!eig_closed(s, l, v, fb.gap)) push_fallback(fb, i);
     orient_largest(v);
     if (evals) {
       evals[i] = l[0];
