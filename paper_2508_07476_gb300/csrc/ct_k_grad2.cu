@@ -357,7 +357,8 @@ __global__ void __launch_bounds__(XT, 512 / XT)
 }
 
 // ---------------------------------------------------------------- z pass
-// One thread per (x, y) column of the output box walks z.  The three partial
+// One thread per column of the output box's (y, x) plane, taken flat (no lane
+// idles at a row's end), walks z.  The three partial
 // fields arrive by 4-byte cp.async into a shared ring of P = 2R+1 steps
 // (dynamic shared memory, P * 3 KB), issued kGzAhead steps ahead; ring slots
 // and register windows are indexed statically because the step loop is
@@ -393,22 +394,21 @@ __device__ __forceinline__ void grad_z_body(const float* __restrict__ F, const B
   // [P] steps of (F0, F1) pairs [kGzThreads][2], then F2 [kGzThreads]: the x and y
   // components run as FP32 pairs (one packed add and fma per tap for both)
   extern __shared__ __align__(16) float gz_ring[];
-  const int tid = threadIdx.y * blockDim.x + threadIdx.x;
-  const int x = ob.lo[0] + blk.x() * blockDim.x + threadIdx.x;
-  const int yr = blk.y() * blockDim.y + threadIdx.y;
-  const bool ok = x < ob.lo[0] + ob.n[0] && yr < ob.n[1];
-  const int xi = min(x, ob.lo[0] + ob.n[0] - 1);
-  const int y = ob.lo[1] + min(yr, ob.n[1] - 1);
+  const int tid = threadIdx.x;
+  // the column: fields and outputs share their (y, x) plane, taken flat
+  const int plane = ob.n[0] * ob.n[1];
+  const unsigned column = blk.x() * kGzThreads + tid;
+  const bool ok = column < (unsigned)plane;
+  const int col = (int)min(column, (unsigned)plane - 1u);
   const int p0 = ob.lo[2] + blk.z() * seg;  // first output plane
   const int L = min(seg, ob.lo[2] + ob.n[2] - p0);
   if (L <= 0) return;
   const int nsteps = L + 2 * RS;
 
-  // input column (xi, y) of the partial fields; step s reads plane p0 - RS + s,
-  // clamped to the planes the fields cover (the volume's edges, or the halo)
+  // step s reads plane p0 - RS + s of the partial fields, clamped to the planes they
+  // cover (the volume's edges, or the halo)
   const int64_t nab = box_vox(ab);
-  const float* base = F + box_index(ab, xi, y, ab.lo[2]);
-  const int plane = ab.n[0] * ab.n[1];
+  const float* base = F + col;
   const int q0 = p0 - RS - ab.lo[2];
   auto src = [&](int s) -> const float* { return base + (int64_t)min(max(q0 + s, 0), ab.n[2] - 1) * plane; };
   const uint32_t ring01 = (uint32_t)__cvta_generic_to_shared(gz_ring + 2 * tid);
@@ -429,9 +429,8 @@ __device__ __forceinline__ void grad_z_body(const float* __restrict__ F, const B
   const int64_t nob = box_vox(ob);
   float* J = static_cast<float*>(Jv);
   __half* Jh = static_cast<__half*>(Jv);
-  const int64_t obase_i = box_index(ob, xi, y, p0);
+  const int64_t obase_i = (int64_t)(p0 - ob.lo[2]) * plane + col;
   float* obase = J + obase_i;
-  const int ostride = ob.n[0] * ob.n[1];
   float2 w01[P];
   float w2[P];
 #pragma unroll
@@ -463,7 +462,7 @@ __device__ __forceinline__ void grad_z_body(const float* __restrict__ F, const B
         float gx = gxy.x, gy = gxy.y;
         if (GOUT) {  // the gradient itself, held in FP16 (scaled) in the mixed form
           if (ok) {
-            const int64_t o = obase_i + (int64_t)(s - 2 * RS) * ostride;
+            const int64_t o = obase_i + (int64_t)(s - 2 * RS) * plane;
             if (MIXED) {
               Jh[o] = __float2half_rn(gx * kGzHalfScale);
               Jh[o + nob] = __float2half_rn(gy * kGzHalfScale);
@@ -482,7 +481,7 @@ __device__ __forceinline__ void grad_z_body(const float* __restrict__ F, const B
           gz = __half2float(__float2half_rn(gz * kGzHalfScale)) * (1.0f / kGzHalfScale);
         }
         if (ok) {
-          float* o = obase + (int64_t)(s - 2 * RS) * ostride;
+          float* o = obase + (int64_t)(s - 2 * RS) * plane;
           if (ps.unit) {
             o[0] = gx * gx;
             o[nob] = gy * gy;
@@ -513,9 +512,7 @@ __global__ void __launch_bounds__(kGzThreads, CT_GZ_MINB > 0 ? CT_GZ_MINB : (RS 
   grad_z_body<RS, MIXED, GOUT>(F, ab, Jv, ob, seg, taps, ps, HwBlock{});
 }
 
-// The same (the six products) over a batch of volumes in one persistent launch,
-// blocks of kGzMultiX x (kGzThreads / kGzMultiX) threads.
-constexpr int kGzMultiX = 128;
+// The same (the six products) over a batch of volumes in one persistent launch.
 template <int RS, bool MIXED>
 __global__ void __launch_bounds__(kGzThreads, CT_GZ_MINB > 0 ? CT_GZ_MINB : (RS <= 8 ? 3 : 2))
     k_grad_z_multi(const GzItem* __restrict__ items, const MultiTable T, const __grid_constant__ Taps taps,
@@ -544,6 +541,9 @@ static size_t gz_smem() {
 template <int RS>
 static cudaError_t prepare_gs() {
   cudaError_t e = set_xy_attr<RS, CT_GXY_XT>();
+  if (e == cudaSuccess) e = set_xy_attr<RS, 64>();
+  if (e == cudaSuccess) e = set_xy_attr<RS, 96>();
+  if (e == cudaSuccess) e = set_xy_attr<RS, 160>();
   const int sm = (int)gz_smem<RS>();
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_grad_xy_multi<RS, CT_GXY_XT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -590,52 +590,69 @@ static cudaError_t launch_gxy_t(const uint16_t* vol, const Box& vb, const int di
                                 const Taps& tx, const Taps& ty, cudaStream_t st) {
   using G = GXYGeom<RS, XT>;
   if (ab.n[2] > 65535) return cudaErrorInvalidValue;
+  static int sms = 1;
+  static const int slots = resident_ctas(k_grad_xy<RS, XT>, XT, G::SMEM, &sms);
   const int64_t ctas = (int64_t)((ab.n[0] + XT - 1) / XT) * ab.n[2];
-  int nseg = 1;
-  while (nseg < 16 && ctas * nseg < (int64_t)152 * 2 * 4 * (256 / XT) && ab.n[1] / (nseg * 2) >= 8 * G::TB) nseg *= 2;
-  const int seg = (ab.n[1] + nseg - 1) / nseg;
+  // a warm-up block stages its rows and filters them along x
+  const int seg = walk_segment(ctas, ab.n[1], G::TB, 0.5 * G::W * G::TB, slots, sms);
   dim3 grid((ab.n[0] + XT - 1) / XT, ab.n[2], (ab.n[1] + seg - 1) / seg);
+  if (grid.z > 65535) return cudaErrorInvalidValue;
   k_grad_xy<RS, XT><<<grid, XT, G::SMEM, st>>>(vol, vb, dims[0], dims[1], F, ab, seg, tx, ty);
   return cudaGetLastError();
 }
 
-// 128-column CTAs at every width: four CTAs of 4 warps per SM wait at their
-// barriers independently (512^3: 0.62 ms, against 0.67 with two CTAs of 256
-// columns, the same 16 warps per SM)
+// The CTA width (columns) that covers a row of n0 with the least work: the
+// columns of its CTAs, idle ones included, and the staged columns beside
+// each CTA's own (halo per side), a staged one weighing `stage` of a column.
+int cta_width(int n0, int halo, double stage, const int* widths, int n) {
+  int best = widths[0];
+  double least = 1e300;
+  for (int i = 0; i < n; ++i) {
+    const int w = widths[i], ctas = (n0 + w - 1) / w;
+    const double cost = (double)ctas * (w + stage * 2 * halo);
+    if (cost < least) least = cost, best = w;
+  }
+  return best;
+}
+
+// 16 warps per SM at every width, in CTAs that wait at their barriers
+// independently (512^3: 128 columns 0.62 ms, against 0.67 with two CTAs of 256).
+// The width that leaves the fewest idle columns: a 173-column row took two CTAs of 128,
+// now two of 96.
 template <int RS>
 static cudaError_t launch_gxy_r(const uint16_t* vol, const Box& vb, const int dims[3], float* F, const Box& ab,
                                 const Taps& tx, const Taps& ty, cudaStream_t st) {
-  return launch_gxy_t<RS, CT_GXY_XT>(vol, vb, dims, F, ab, tx, ty, st);
+  static const int widths[] = {CT_GXY_XT, 96, 64, 160};
+  switch (cta_width(ab.n[0], GXYGeom<RS, CT_GXY_XT>::XA, 0.3, widths, 4)) {
+    case 64: return launch_gxy_t<RS, 64>(vol, vb, dims, F, ab, tx, ty, st);
+    case 96: return launch_gxy_t<RS, 96>(vol, vb, dims, F, ab, tx, ty, st);
+    case 160: return launch_gxy_t<RS, 160>(vol, vb, dims, F, ab, tx, ty, st);
+    default: return launch_gxy_t<RS, CT_GXY_XT>(vol, vb, dims, F, ab, tx, ty, st);
+  }
+}
+
+template <int RS, bool MIXED, bool GOUT>
+static cudaError_t launch_gz_t(const float* F, const Box& ab, void* J, const Box& ob, const Taps& taps,
+                               const ProdScale& ps, cudaStream_t st) {
+  static int sms = 1;
+  static const int slots = resident_ctas(k_grad_z<RS, MIXED, GOUT>, kGzThreads, gz_smem<RS>(), &sms);
+  const int blocks = (ob.n[0] * ob.n[1] + kGzThreads - 1) / kGzThreads;
+  // a warm-up step loads and computes nothing
+  const int seg = walk_segment(blocks, ob.n[2], 1, 0.4 * (2 * RS), slots, sms);
+  const dim3 grid(blocks, 1, (ob.n[2] + seg - 1) / seg);
+  if (grid.z > 65535) return cudaErrorInvalidValue;
+  k_grad_z<RS, MIXED, GOUT><<<grid, kGzThreads, gz_smem<RS>(), st>>>(F, ab, J, ob, seg, taps, ps);
+  return cudaGetLastError();
 }
 
 template <int RS>
 static cudaError_t launch_gz_r(const float* F, const Box& ab, void* J, const Box& ob, const Taps& taps,
                                const ProdScale& ps, bool mixed, bool gout, cudaStream_t st) {
-  // warps along x: the widest that leaves the fewest idle columns
-  int wx = 1;
-  for (int w = 2; w <= kGzThreads / 32; w *= 2) {
-    const int span = 32 * w, best = 32 * wx;
-    if (32 * (w / 2) >= ob.n[0]) break;
-    if ((ob.n[0] + span - 1) / span * span <= (ob.n[0] + best - 1) / best * best) wx = w;
-  }
-  dim3 block(32 * wx, kGzThreads / (32 * wx));
-  const int64_t cols = (int64_t)((ob.n[0] + block.x - 1) / block.x) * ((ob.n[1] + block.y - 1) / block.y);
-  int nseg = 1;
-  while (nseg < 16 && cols * nseg < (int64_t)152 * 2 * 4 && ob.n[2] / (nseg * 2) >= 4 * (2 * RS + 1)) nseg *= 2;
-  const int seg = (ob.n[2] + nseg - 1) / nseg;
-  dim3 grid((ob.n[0] + block.x - 1) / block.x, (ob.n[1] + block.y - 1) / block.y, (ob.n[2] + seg - 1) / seg);
-  if (grid.y > 65535 || grid.z > 65535) return cudaErrorInvalidValue;
-  if (gout) {
-    if (mixed)
-      k_grad_z<RS, true, true><<<grid, block, gz_smem<RS>(), st>>>(F, ab, J, ob, seg, taps, ps);
-    else
-      k_grad_z<RS, false, true><<<grid, block, gz_smem<RS>(), st>>>(F, ab, J, ob, seg, taps, ps);
-  } else if (mixed) {
-    k_grad_z<RS, true, false><<<grid, block, gz_smem<RS>(), st>>>(F, ab, J, ob, seg, taps, ps);
-  } else {
-    k_grad_z<RS, false, false><<<grid, block, gz_smem<RS>(), st>>>(F, ab, J, ob, seg, taps, ps);
-  }
-  return cudaGetLastError();
+  if (gout)
+    return mixed ? launch_gz_t<RS, true, true>(F, ab, J, ob, taps, ps, st)
+                 : launch_gz_t<RS, false, true>(F, ab, J, ob, taps, ps, st);
+  return mixed ? launch_gz_t<RS, true, false>(F, ab, J, ob, taps, ps, st)
+               : launch_gz_t<RS, false, false>(F, ab, J, ob, taps, ps, st);
 }
 
 cudaError_t launch_grad_xy(const uint16_t* vol, const Box& vb, const int dims[3], float* F, const Box& ab,
@@ -700,9 +717,8 @@ cudaError_t launch_grad_xy_multi(const GxyItem* items, const MultiTable& T, int6
 template <int RS>
 static uint3 gz_item(GzItem& it) {
   const Box& ob = it.ob;
-  const dim3 block(kGzMultiX, kGzThreads / kGzMultiX);
   it.seg = ob.n[2];  // unsplit (see gxy_item)
-  return make_uint3((ob.n[0] + block.x - 1) / block.x, (ob.n[1] + block.y - 1) / block.y, 1);
+  return make_uint3((ob.n[0] * ob.n[1] + kGzThreads - 1) / kGzThreads, 1, 1);
 }
 
 uint3 grad_z_item(int rk, GzItem& it) {
@@ -719,7 +735,7 @@ uint3 grad_z_item(int rk, GzItem& it) {
 template <int RS>
 static cudaError_t gz_multi(const GzItem* items, const MultiTable& T, int64_t blocks, const Taps& tz,
                             const ProdScale& ps, bool mixed, cudaStream_t st) {
-  const dim3 block(kGzMultiX, kGzThreads / kGzMultiX);
+  const int block = kGzThreads;
   if (mixed) {
     const int grid = persistent_grid(k_grad_z_multi<RS, true>, kGzThreads, gz_smem<RS>(), blocks);
     k_grad_z_multi<RS, true><<<grid, block, gz_smem<RS>(), st>>>(items, T, tz, ps);

@@ -28,8 +28,7 @@ namespace ct {
 constexpr int kStages = 3;      // cp.async ring depth (blocks)
 static_assert(CT_XY_TB == 8 || CT_XY_TB == 16, "rows per block");
 
-// XT output columns per CTA (= threads): 256, or 128 for widths that 256
-// would cover with a mostly idle last CTA.
+// XT output columns per CTA (= threads), 512 / XT CTAs per SM.
 template <int RR, int XT>
 struct XYGeom {
   // rows per block: 8 for the widest kernels, whose y window would not fit
@@ -380,7 +379,7 @@ __global__ void __launch_bounds__(XT, CT_XY_MINB * 256 / XT)
   });
 }
 
-template <int RR, int XT>
+template <int RR, int XT, bool SAME>
 static cudaError_t launch_xy_rt(const float* in, const Box& ib, const int dims[3], float* out, const Box& ob,
                                 const Taps& tx, const Taps& ty, cudaStream_t st) {
   using G = XYGeom<RR, XT>;
@@ -389,14 +388,13 @@ static cudaError_t launch_xy_rt(const float* in, const Box& ib, const int dims[3
   const int64_t rows = (int64_t)6 * ob.n[2];
   if (rows > 65535) return cudaErrorInvalidValue;
   const int64_t ctas = (int64_t)((ob.n[0] + XT - 1) / XT) * rows;
-  int nseg = 1;
-  while (nseg < 16 && ctas * nseg < (int64_t)152 * 2 * 4 * (256 / XT) && ob.n[1] / (nseg * 2) >= 8 * kTB) nseg *= 2;
-  const int seg = (ob.n[1] + nseg - 1) / nseg;
+  static int sms = 1;
+  static const int slots = resident_ctas(k_rho_xy<RR, XT, SAME>, XT, smem, &sms);
+  // a warm-up block stages its rows and filters them along x
+  const int seg = walk_segment(ctas, ob.n[1], kTB, 0.6 * G::W * kTB, slots, sms);
   dim3 grid((ob.n[0] + XT - 1) / XT, (unsigned)rows, (ob.n[1] + seg - 1) / seg);
-  if (std::memcmp(&tx, &ty, sizeof(Taps)) == 0)
-    k_rho_xy<RR, XT, true><<<grid, XT, smem, st>>>(in, ib, dims[0], dims[1], out, ob, seg, tx, ty);
-  else
-    k_rho_xy<RR, XT, false><<<grid, XT, smem, st>>>(in, ib, dims[0], dims[1], out, ob, seg, tx, ty);
+  if (grid.z > 65535) return cudaErrorInvalidValue;
+  k_rho_xy<RR, XT, SAME><<<grid, XT, smem, st>>>(in, ib, dims[0], dims[1], out, ob, seg, tx, ty);
   return cudaGetLastError();
 }
 
@@ -410,17 +408,38 @@ template <int RR>
 static cudaError_t launch_xy_r(const float* in, const Box& ib, const int dims[3], float* out, const Box& ob,
                                const Taps& tx, const Taps& ty, cudaStream_t st) {
   if (box_vox(ib) >= ((int64_t)1 << 31) || box_vox(ob) >= ((int64_t)1 << 31)) return cudaErrorInvalidValue;
-  return narrow_xy(ob.n[0]) ? launch_xy_rt<RR, 128>(in, ib, dims, out, ob, tx, ty, st)
-                            : launch_xy_rt<RR, 256>(in, ib, dims, out, ob, tx, ty, st);
+  if (std::memcmp(&tx, &ty, sizeof(Taps)) != 0)  // anisotropic voxels: two tap sets
+    return narrow_xy(ob.n[0]) ? launch_xy_rt<RR, 128, false>(in, ib, dims, out, ob, tx, ty, st)
+                              : launch_xy_rt<RR, 256, false>(in, ib, dims, out, ob, tx, ty, st);
+  // the width with the fewest idle columns (they filter like the others); a staged
+  // column beside the CTA's own costs a tenth of one (0.02 .. 0.25 choose alike
+  // but for narrow rows): 173 columns in two CTAs of 96 instead of one of 256
+  static const int widths[] = {256, 128, 96, 64, 160};
+  switch (cta_width(ob.n[0], RR, 0.1, widths, 5)) {
+    case 64: return launch_xy_rt<RR, 64, true>(in, ib, dims, out, ob, tx, ty, st);
+    case 96: return launch_xy_rt<RR, 96, true>(in, ib, dims, out, ob, tx, ty, st);
+    case 128: return launch_xy_rt<RR, 128, true>(in, ib, dims, out, ob, tx, ty, st);
+    case 160: return launch_xy_rt<RR, 160, true>(in, ib, dims, out, ob, tx, ty, st);
+    default: return launch_xy_rt<RR, 256, true>(in, ib, dims, out, ob, tx, ty, st);
+  }
+}
+
+template <int RR, int XT>
+constexpr int xy_smem() {
+  using G = XYGeom<RR, XT>;
+  return (int)(sizeof(float) * (kStages * G::TB * G::XS + G::TB * G::SXS));
+}
+
+template <int RR, int XT, bool SAME>
+static cudaError_t prepare_xy_1() {
+  return cudaFuncSetAttribute(k_rho_xy<RR, XT, SAME>, cudaFuncAttributeMaxDynamicSharedMemorySize, xy_smem<RR, XT>());
 }
 
 template <int RR, int XT>
 static cudaError_t prepare_xy_rt() {
-  using G = XYGeom<RR, XT>;
-  const int smem = (int)(sizeof(float) * (kStages * G::TB * G::XS + G::TB * G::SXS));
-  cudaError_t e = cudaFuncSetAttribute(k_rho_xy<RR, XT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_rho_xy<RR, XT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  constexpr int smem = xy_smem<RR, XT>();
+  cudaError_t e = prepare_xy_1<RR, XT, true>();
+  if (e == cudaSuccess) e = prepare_xy_1<RR, XT, false>();
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_rho_xy_multi<RR, XT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e == cudaSuccess)
@@ -432,6 +451,9 @@ template <int RR>
 static cudaError_t prepare_xy_r() {
   cudaError_t e = prepare_xy_rt<RR, 256>();
   if (e == cudaSuccess) e = prepare_xy_rt<RR, 128>();
+  if (e == cudaSuccess) e = prepare_xy_1<RR, 64, true>();
+  if (e == cudaSuccess) e = prepare_xy_1<RR, 96, true>();
+  if (e == cudaSuccess) e = prepare_xy_1<RR, 160, true>();
   return e;
 }
 

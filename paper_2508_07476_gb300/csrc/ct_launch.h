@@ -13,6 +13,54 @@ namespace ct {
 cudaError_t prepare_rho_xy_kernels();
 cudaError_t prepare_grad_split_kernels();
 
+// How many segments to cut the walk of a streaming kernel into: `ctas` CTAs
+// walk n positions each, a segment of L of them costing L + warm (warm: the
+// steps before its first output, in steps of the walk), and `slots` CTAs are
+// resident at once on `sms` SMs.  The cheapest of up to 64 cuts, whole waves
+// of CTAs counted as they run side by side, the last one by the CTAs per SM it
+// still holds but no less than kLoneCta of a full wave (a lone CTA waits for
+// its own loads and barriers).  seg: a multiple of unit.  Before, the walks were
+// cut by powers of two while the grid was below a fixed size and a segment
+// above a fixed length, so a 64^3 volume ran grad_z in 16 CTAs: its gradient
+// x/y, z and rho z passes 15.4, 16.4, 10.4 us, and 10.8, 8.3, 8.1 now;
+// 173 x 141 x 118: gradient 39.8 + 37.6 us, and 25.8 + 20.5 now.  The times are
+// flat in the weights: kLoneCta 0.25 .. 0.8 and warm x 0.6 .. 1.5 move none of the
+// measured volumes by more than 1%.
+constexpr double kLoneCta = 0.5;
+inline int walk_segment(int64_t ctas, int n, int unit, double warm, int slots, int sms) {
+  double best = 1e300;
+  int best_seg = n;
+  for (int s = 1; s <= 64; ++s) {
+    const int seg = ((n + s - 1) / s + unit - 1) / unit * unit;
+    const int64_t total = ctas * ((n + seg - 1) / seg);
+    const int64_t full = total / slots, rest = total - full * slots;
+    double waves = (double)full;
+    if (rest) {
+      const double r = (double)((rest + sms - 1) / sms) * sms / slots;
+      waves += r > kLoneCta ? (r < 1.0 ? r : 1.0) : kLoneCta;
+    }
+    const double cost = waves * (seg + warm);
+    if (cost < best * 0.99) best = cost, best_seg = seg;  // a finer cut only where it gains
+    if (seg <= unit) break;
+  }
+  return best_seg;
+}
+
+// The CTA width (columns) of the kernels that walk along y: of `widths`, the
+// first that covers a row of n0 with the least work.
+int cta_width(int n0, int halo, double stage, const int* widths, int n);
+
+// CTAs of a kernel resident at once on the current device (its SM count in *sms).
+template <typename K>
+int resident_ctas(K kernel, int threads, size_t smem, int* sms) {
+  int dev = 0, per = 1;
+  *sms = 1;
+  cudaGetDevice(&dev);
+  if (cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || *sms < 1) *sms = 1;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, threads, smem) != cudaSuccess || per < 1) per = 1;
+  return per * *sms;
+}
+
 // Instantiated radius that serves radius r (zero taps pad the difference), or -1.
 int sigma_kernel_radius(int r);
 int rho_kernel_radius(int r);
