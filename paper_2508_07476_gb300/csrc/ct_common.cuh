@@ -118,9 +118,16 @@ __device__ __forceinline__ void for_each_vblock(const MultiTable& T, F&& f) {
   }
 }
 
-// Asynchronous 4-byte global -> shared copies (cp.async), grouped per commit.
+// The CTA's barrier, for kernels whose warps reach it from different loops (every
+// warp as often; __syncthreads() wants one place for all).
+__device__ __forceinline__ void cta_barrier() { asm volatile("bar.sync 0;" ::: "memory"); }
+
+// Asynchronous 4- and 8-byte global -> shared copies (cp.async), grouped per commit.
 __device__ __forceinline__ void cp_async4(uint32_t smem_dst, const float* gsrc) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(smem_dst), "l"(gsrc) : "memory");
+}
+__device__ __forceinline__ void cp_async8(uint32_t smem_dst, const float* gsrc) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(smem_dst), "l"(gsrc) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 template <int N>

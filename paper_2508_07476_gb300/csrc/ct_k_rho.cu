@@ -322,12 +322,144 @@ dim3 rho_stream_block(const Box& ob, int axis) {
   return dim3(32 * wx, kStreamThreads / (32 * wx));
 }
 
+// ------------------------------------------------------ z pass on column pairs
+// Along z the columns of a component are its whole (y, x) plane, so they are taken
+// flat: no lane idles at a row's end.  A thread walks two neighbouring columns
+// (8-byte copies; the plane's rows are even) with a window of pairs, and every
+// tap is one packed FMA on the pair (each half rounded as the scalar FMA, in
+// the same order, so the results are those of rho_stream_body to the bit).  A packed
+// FMA takes the issue slots of two (measured: the FMA rate is that of scalar
+// ones, 37 TFMA/s, and integer work beside either adds to its time), so it only
+// spares the address and copy work that both columns share, which matters: the
+// scalar form issued 48% more instructions than FMAs.  The taps are the outer
+// loop (one load per tap and kZ2Outputs outputs) and symmetric, so half of them
+// are read.  250 x 203 x 190, R = 24: 157 us with a thread per column, 119 us
+// now (61 us at the copy rate for its 412 MB, 76 us at the FMA rate).
+constexpr int kZ2Threads = 128;
+constexpr int kZ2Outputs = 8;  // per column and block of the walk
+
+// in: planes of in_plane elements (rows of in_row); out: rows of out_row, the first
+// out_row columns of each input row.  DENSE8: out rows are even and 8-byte aligned.
+template <int RR, bool DENSE8>
+__global__ void __launch_bounds__(kZ2Threads, RR >= 32 ? 2 : 3)
+    k_rho_z2(const float* __restrict__ in, int64_t in_vox, int a_in, int n_in, int dimz, int in_row, int in_plane,
+             float* __restrict__ out, int64_t out_vox, int a_out, int n_out, int out_row, int out_plane, int seg,
+             const __grid_constant__ Taps taps) {
+  constexpr int kT = kZ2Outputs;
+  constexpr int WN = kT + 2 * RR;
+  __shared__ __align__(16) float2 ring[2 * kT][kZ2Threads];
+  const int t = threadIdx.x;
+  const unsigned c = 2u * (blockIdx.x * kZ2Threads + t);  // the pair's first column
+  const bool in_range = c < (unsigned)in_plane;
+  const int c0 = in_range ? (int)c : in_plane - 2;  // even: pairs past the plane read the last one
+  const int y = c0 / in_row, x = c0 - y * in_row;
+  const bool ok0 = in_range && x < out_row, ok1 = in_range && x + 1 < out_row;
+  const int p0 = a_out + blockIdx.z * seg;
+  const int L = min(seg, a_out + n_out - p0);
+  if (L <= 0) return;
+  const float* base = in + blockIdx.y * in_vox + c0;
+  const int qlo = max(0, a_in) - a_in, qhi = min(dimz - 1, a_in + n_in - 1) - a_in;
+  const int q0 = p0 - RR - a_in;
+  auto src = [&](int step) -> const float* { return base + min(max(q0 + step, qlo), qhi) * in_plane; };
+  float* o = out + blockIdx.y * out_vox + (p0 - a_out) * out_plane + y * out_row + x;
+  const uint32_t ring0 = (uint32_t)__cvta_generic_to_shared(&ring[0][t]);
+  constexpr uint32_t kSlot = kZ2Threads * sizeof(float2);
+  auto w2 = [&](int k) {  // tap k = tap 2 RR - k, on both columns
+    const float w = taps.w[k <= RR ? k : 2 * RR - k];
+    return make_float2(w, w);
+  };
+  float2 win[WN];
+#pragma unroll
+  for (int j = 0; j < 2 * RR; ++j) win[j] = __ldg(reinterpret_cast<const float2*>(src(j)));
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+#pragma unroll
+    for (int u = 0; u < kT; ++u) cp_async8(ring0 + (h * kT + u) * kSlot, src(2 * RR + h * kT + u));
+    cp_async_commit();
+  }
+  const int nb = (L + kT - 1) / kT;
+  for (int bk = 0; bk < nb; ++bk) {
+    cp_async_wait<1>();  // block bk has landed (this thread's own copies)
+    const int half = (bk & 1) * kT;
+#pragma unroll
+    for (int u = 0; u < kT; ++u) win[2 * RR + u] = ring[half + u][t];
+    // two chains per output, even and odd taps
+    float2 a0[kT], a1[kT];
+#pragma unroll
+    for (int i = 0; i < kT; ++i) a0[i] = __fmul2_rn(w2(0), win[i]);
+#pragma unroll
+    for (int i = 0; i < kT; ++i) a1[i] = __fmul2_rn(w2(1), win[i + 1]);
+#pragma unroll
+    for (int k = 2; k <= 2 * RR; k += 2) {
+#pragma unroll
+      for (int i = 0; i < kT; ++i) a0[i] = __ffma2_rn(w2(k), win[i + k], a0[i]);
+      if (k + 1 <= 2 * RR) {
+#pragma unroll
+        for (int i = 0; i < kT; ++i) a1[i] = __ffma2_rn(w2(k + 1), win[i + k + 1], a1[i]);
+      }
+    }
+    const int s0 = bk * kT;
+#pragma unroll
+    for (int i = 0; i < kT; ++i) {
+      const float2 r = __fadd2_rn(a0[i], a1[i]);
+      if (s0 + i < L) {
+        float* q = o + (s0 + i) * out_plane;
+        if (DENSE8) {
+          if (ok0) *reinterpret_cast<float2*>(q) = r;
+        } else {
+          if (ok0) q[0] = r.x;
+          if (ok1) q[1] = r.y;
+        }
+      }
+    }
+    // refill the slots just consumed with block bk + 2
+#pragma unroll
+    for (int u = 0; u < kT; ++u) cp_async8(ring0 + (half + u) * kSlot, src(2 * RR + (bk + 2) * kT + u));
+    cp_async_commit();
+#pragma unroll
+    for (int j = 0; j < 2 * RR; ++j) win[j] = win[j + kT];
+  }
+  cp_async_wait<0>();
+}
+
+template <int RR, bool DENSE8>
+static cudaError_t launch_z2_t(const float* in, const Box& ib, int dimz, float* out, const Box& ob, const Taps& taps,
+                               cudaStream_t st) {
+  static int sms = 1;
+  static const int slots = resident_ctas(k_rho_z2<RR, DENSE8>, kZ2Threads, 0, &sms);
+  const int plane = ib.n[0] * ib.n[1];
+  const int blocks = (plane / 2 + kZ2Threads - 1) / kZ2Threads;
+  // a warm-up step loads one pair and computes nothing
+  const int seg = walk_segment((int64_t)blocks * 6, ob.n[2], kZ2Outputs, 0.25 * (2 * RR), slots, sms);
+  dim3 grid(blocks, 6, (ob.n[2] + seg - 1) / seg);
+  if (grid.z > 65535) return cudaErrorInvalidValue;
+  k_rho_z2<RR, DENSE8><<<grid, kZ2Threads, 0, st>>>(in, box_vox(ib), ib.lo[2], ib.n[2], dimz, ib.n[0], plane, out,
+                                                    box_vox(ob), ob.lo[2], ob.n[2], ob.n[0], ob.n[0] * ob.n[1], seg,
+                                                    taps);
+  return cudaGetLastError();
+}
+
+// Whether k_rho_z2 takes the z pass: the output's columns are the first ones of
+// the input's rows, and the input's rows are even (a thread's pair is one row's).
+static bool z2_ok(const float* in, const Box& ib, const Box& ob) {
+  return ib.lo[0] == ob.lo[0] && ib.lo[1] == ob.lo[1] && ib.n[1] == ob.n[1] && ib.n[0] >= ob.n[0] &&
+         ib.n[0] % 2 == 0 && (uintptr_t)in % 8 == 0;
+}
+
+template <int RR>
+static cudaError_t launch_z2_r(const float* in, const Box& ib, int dimz, float* out, const Box& ob, const Taps& taps,
+                               cudaStream_t st) {
+  return ob.n[0] % 2 == 0 && (uintptr_t)out % 8 == 0 ? launch_z2_t<RR, true>(in, ib, dimz, out, ob, taps, st)
+                                                     : launch_z2_t<RR, false>(in, ib, dimz, out, ob, taps, st);
+}
+
 template <int RR>
 static cudaError_t launch_stream_r(const float* in, const Box& ib, const int dims[3], float* out, const Box& ob,
                                    int axis, const Taps& taps, int block_t, cudaStream_t st) {
   const int other = 3 - axis;
   const int n_axis = ob.n[axis];
   if (box_vox(ib) >= ((int64_t)1 << 31) || box_vox(ob) >= ((int64_t)1 << 31)) return cudaErrorInvalidValue;
+  if (axis == 2 && z2_ok(in, ib, ob)) return launch_z2_r<RR>(in, ib, dims[2], out, ob, taps, st);
   const int seg = stream_seg(ob, axis, RR);
   const dim3 block = rho_stream_block(ob, axis);
   dim3 grid((ob.n[0] + block.x - 1) / block.x, (6 * ob.n[other] + block.y - 1) / block.y, (n_axis + seg - 1) / seg);
