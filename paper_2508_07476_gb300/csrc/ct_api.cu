@@ -453,13 +453,49 @@ bool use_tc(const ct_plan P, const Scale& sc, const int dims[3], int axis) {
 //   - otherwise the products J and the x, y passes (tensor cores per axis, or
 //     the fused FP32 stencil), then the z pass:
 //       grad_xy -> B, grad_z: J -> A, x / y -> B or A, z -> out.
+// The scratch rows of the chain are padded to multiples of 8 elements, and its
+// haloed boxes start on multiples of 8 where they start inside the volume, so that
+// every row of every intermediate starts on a 32-byte sector and is read with
+// 16-byte copies whatever the volume's width (a ragged one otherwise goes
+// element by element through the rho passes: a 173 x 141 x 118 crop at R = 16, rho
+// x/y 118 and z 47 us, 90 and 33 us padded and with the CTA widths to fit).  The columns added lie beyond what any output reads; they hold
+// values of clamped coordinates.  Not for narrow boxes, where the padding would be a
+// large share, nor where it would push the planes past 32-bit indices.
+constexpr int kPadX = 8, kPadMinX = 64;
+
+struct ChainBoxes {
+  Box G;   // the gradient and the products: ob grown by R(rho)
+  Box Ab;  // the gradient's partial fields: G grown by R(sigma) in z
+  Box S;   // the tensor, when it stays in scratch
+  int64_t need;  // voxels per scratch buffer
+};
+
+ChainBoxes chain_boxes(const Scale& sc, const int dims[3], const Box& vb, const Box& ob) {
+  ChainBoxes c;
+  c.G = grow_clip3(ob, sc.rr, dims);
+  c.S = ob;
+  Box g = c.G;
+  g.lo[0] = g.lo[0] / kPadX * kPadX;
+  g.n[0] = (c.G.lo[0] + c.G.n[0] - g.lo[0] + kPadX - 1) / kPadX * kPadX;
+  if (ob.n[0] >= kPadMinX && 6 * box_vox(g) < (int64_t(1) << 31) &&
+      box_vox(grad_partial_box(g, vb, sc.rks, dims[2])) < (int64_t(1) << 31)) {
+    c.G = g;
+    c.S.n[0] = (ob.n[0] + kPadX - 1) / kPadX * kPadX;
+  }
+  // the gradient keeps its 3 partial planes (over G grown in z) in one buffer of 6 planes
+  c.Ab = grad_partial_box(c.G, vb, sc.rks, dims[2]);
+  c.need = std::max<int64_t>(box_vox(c.G), (box_vox(c.Ab) + 1) / 2);
+  return c;
+}
+
 ct_status smooth_chain(ct_plan P, const Scale& sc, const int dims[3], const uint16_t* vol, const Box& vb,
-                       const Box& ob, int slot, bool mixed, cudaStream_t st, float* S_out, float** S_res) {
-  const Box G = grow_clip3(ob, sc.rr, dims);
-  // the gradient keeps its 3 partial planes (over G grown in z) in B
-  const Box Ab = grad_partial_box(G, vb, sc.rks, dims[2]);
-  const int64_t need = std::max<int64_t>(box_vox(G), (box_vox(Ab) + 1) / 2);
-  ct_status rc = ensure_scratch(P, slot, need);
+                       const Box& ob, int slot, bool mixed, cudaStream_t st, float* S_out, float** S_res,
+                       Box* S_box) {
+  const ChainBoxes cb = chain_boxes(sc, dims, vb, ob);
+  const Box &G = cb.G, &Ab = cb.Ab;
+  const Box So = S_out ? ob : cb.S;  // a caller's tensor is dense
+  *S_box = So;
+  ct_status rc = ensure_scratch(P, slot, cb.need);
   if (rc) return rc;
   float* A = P->buf[slot][0];
   float* B = P->buf[slot][1];
@@ -483,14 +519,14 @@ ct_status smooth_chain(ct_plan P, const Scale& sc, const int dims[3], const uint
               "rho z kernel launch");
     CT_LAUNCH(P, st, "rho_y_tc", launch_rho_tc(B, Bz, dims, A, Bzy, 1, sc.tr[1], sc.rkr, ctl, st),
               "rho y kernel launch");
-    CT_LAUNCH(P, st, "rho_x_tc", launch_rho_tc(A, Bzy, dims, S, ob, 0, sc.tr[0], sc.rkr, ctl, st),
+    CT_LAUNCH(P, st, "rho_x_tc", launch_rho_tc(A, Bzy, dims, S, So, 0, sc.tr[0], sc.rkr, ctl, st),
               "rho x kernel launch");
     *S_res = S;
     return CT_OK;
   }
   Box Bx = G, Bxy = G;
   Bx.lo[0] = Bxy.lo[0] = ob.lo[0];
-  Bx.n[0] = Bxy.n[0] = ob.n[0];
+  Bx.n[0] = Bxy.n[0] = cb.S.n[0];
   Bxy.lo[1] = ob.lo[1];
   Bxy.n[1] = ob.n[1];
   CT_LAUNCH(P, st, "grad_z", launch_grad_z(B, Ab, A, G, sc.ts[2], sc.ss, sc.rks, mixed, false, st),
@@ -518,10 +554,10 @@ ct_status smooth_chain(ct_plan P, const Scale& sc, const int dims[3], const uint
   }
   float* S = S_out ? S_out : (Sxy == A ? B : A);
   if (tcz)
-    CT_LAUNCH(P, st, "rho_z_tc", launch_rho_tc(Sxy, Bxy, dims, S, ob, 2, sc.tr[2], sc.rkr, ctl, st),
+    CT_LAUNCH(P, st, "rho_z_tc", launch_rho_tc(Sxy, Bxy, dims, S, So, 2, sc.tr[2], sc.rkr, ctl, st),
               "rho z kernel launch");
   else
-    CT_LAUNCH(P, st, "rho_z", launch_rho_stream(Sxy, Bxy, dims, S, ob, 2, sc.tr[2], sc.rkr, sblock, st),
+    CT_LAUNCH(P, st, "rho_z", launch_rho_stream(Sxy, Bxy, dims, S, So, 2, sc.tr[2], sc.rkr, sblock, st),
               "rho z kernel launch");
   *S_res = S;
   return CT_OK;
@@ -531,10 +567,11 @@ ct_status smooth_chain(ct_plan P, const Scale& sc, const int dims[3], const uint
 ct_status tensor_stages(ct_plan P, const Scale& sc, const int dims[3], const uint16_t* vol, const Box& vb,
                         const Box& ob, float* S_out, int slot, bool mixed, cudaStream_t st) {
   float* S = nullptr;
-  return smooth_chain(P, sc, dims, vol, vb, ob, slot, mixed, st, S_out, &S);
+  Box sb;
+  return smooth_chain(P, sc, dims, vol, vb, ob, slot, mixed, st, S_out, &S, &sb);
 }
 
-ct_status eig_stage(ct_plan P, const float* S, const Box& ob, const uint8_t* mask, const Box& mb, const Frame& F,
+ct_status eig_stage(ct_plan P, const float* S, const Box& sb, const Box& ob, const uint8_t* mask, const Box& mb, const Frame& F,
                     const EigOut& o, int slot, bool mixed, bool compact, cudaStream_t st);
 
 // The fused hot path (Figure 1b, c): gradient and products, the three rho
@@ -544,23 +581,24 @@ ct_status fused_stages(ct_plan P, const Scale& sc, const int dims[3], const uint
                        const Box& ob, const uint8_t* mask, const Box& mb, const Frame& F, const EigOut& o, int slot,
                        bool mixed, cudaStream_t st) {
   float* S = nullptr;
-  ct_status rc = smooth_chain(P, sc, dims, vol, vb, ob, slot, mixed, st, nullptr, &S);
+  Box sb;
+  ct_status rc = smooth_chain(P, sc, dims, vol, vb, ob, slot, mixed, st, nullptr, &S, &sb);
   if (rc) return rc;
   const auto* t = tuned(P, sc, dims);
-  return eig_stage(P, S, ob, mask, mb, F, o, slot, mixed, t && t->eig_compact >= 0 ? t->eig_compact != 0 : P->eig_compact,
+  return eig_stage(P, S, sb, ob, mask, mb, F, o, slot, mixed, t && t->eig_compact >= 0 ? t->eig_compact != 0 : P->eig_compact,
                    st);
 }
 
-// Eigen + angles over ob from S (over ob); outputs in arrays covering o.ab.
-ct_status eig_stage(ct_plan P, const float* S, const Box& ob, const uint8_t* mask, const Box& mb, const Frame& F,
+// Eigen + angles over ob from S (over sb); outputs in arrays covering o.ab.
+ct_status eig_stage(ct_plan P, const float* S, const Box& sb, const Box& ob, const uint8_t* mask, const Box& mb, const Frame& F,
                     const EigOut& o, int slot, bool mixed, bool compact, cudaStream_t st) {
   Fallback fb = fallback_of(P, slot);
   CT_CUDA(cudaMemsetAsync(fb.count, 0, sizeof(int), st), "counter reset");
   CT_LAUNCH(P, st, "eig_angles",
-            launch_eig_angles(S, ob, ob, mask, mb, F, P->p.fill_value, o, mixed, fb, compact, st),
+            launch_eig_angles(S, sb, ob, mask, mb, F, P->p.fill_value, o, mixed, fb, compact, st),
             "eigen kernel launch");
   CT_LAUNCH(P, st, "eig_resolve",
-            launch_eig_angles_fallback(S, ob, ob, mask, mb, F, P->p.fill_value, o, mixed, fb, box_vox(ob), st),
+            launch_eig_angles_fallback(S, sb, ob, mask, mb, F, P->p.fill_value, o, mixed, fb, box_vox(ob), st),
             "re-solve kernel launch");
   return CT_OK;
 }
@@ -1433,7 +1471,7 @@ ct_status run_device_batch(ct_plan P, const ct_item* items, int n, cudaStream_t 
   for (int i = 0; i < n; ++i) total += box_vox(ctx[i].whole);
   for (size_t r = 0; r < rest.size(); ++r) {
     const int i = rest[r], k = k0 + (int)(r % kn);
-    gmax[k] = std::max(gmax[k], box_vox(grow_clip3(ctx[i].whole, ctx[i].sc.rr, ctx[i].dims)));
+    gmax[k] = std::max(gmax[k], chain_boxes(ctx[i].sc, ctx[i].dims, ctx[i].whole, ctx[i].whole).need);
   }
   for (int k = 0; k < K; ++k) {
     if ((rc = ensure_stream(P, k))) return rc;

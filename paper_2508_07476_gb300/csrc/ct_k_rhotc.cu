@@ -1014,7 +1014,9 @@ struct TcLaunch {
     // warps whose 32 lines all lie in the box; x: the windows)
     const int lq = PROD == 2 ? 8 : 4;  // elements per 16 bytes
     const bool rows16 = ((uintptr_t)in % 16) == 0 && ib.n[0] % lq == 0;
-    const bool vin = axis == 0 ? rows16 && ib.lo[0] % 4 == 0 : rows16 && (ob.lo[0] - ib.lo[0]) % lq == 0;
+    // (the x form's last piece ends at the volume's edge, which padded rows may run past)
+    const bool vin = axis == 0 ? rows16 && ib.lo[0] % 4 == 0 && std::min(dims[0], ib.lo[0] + ib.n[0]) % 4 == 0
+                               : rows16 && (ob.lo[0] - ib.lo[0]) % lq == 0;
     const bool vout = axis == 0 && ((uintptr_t)out % 16) == 0 && ob.n[0] % 4 == 0 && ob.lo[0] % 4 == 0;
     int flags = (vin ? 1 : 0) | (vout ? 2 : 0);
     // x form: tensor maps when each 128-row group is 128 consecutive rows of one component,

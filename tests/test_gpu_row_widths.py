@@ -1,0 +1,69 @@
+"""Row widths around every boundary of the stencil chain's work splitting: the
+padding of scratch rows (from 64 columns on, to multiples of 8), the CTA widths of the
+x/y kernels (64, 96, 128, 160, 256 columns), odd and even planes of the z
+passes, walks cut into segments, and boxes whose haloed rows start anywhere.
+The stage's tensor against the FP64 oracle, and every box equal to the whole
+volume bit for bit."""
+import numpy as np
+import pytest
+
+from oracle import oracle as O
+from paper_2508_07476_gb300 import _lib, build
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+import gpu_util as G  # noqa: E402
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _ready():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    build.build()
+    _lib.load()
+
+
+def _vol(shape, seed):
+    import scipy.ndimage as ndi
+    rng = np.random.default_rng(seed)
+    v = ndi.gaussian_filter(rng.integers(500, 3000, size=shape).astype(np.float64), 1.0)
+    return np.clip(np.rint(v + rng.normal(0, 30, size=shape)), 0, 65535).astype(np.uint16)
+
+
+@pytest.mark.parametrize("nx", [31, 63, 64, 65, 72, 95, 97, 129, 161, 193, 255, 257, 321])
+@pytest.mark.parametrize("sigma,rho", [(1.0, 2.0), (0.7, 1.5), (2.0, 6.0)])
+def test_tensor_of_every_row_width(nx, sigma, rho):
+    shape = (7, 23, nx) if nx % 2 else (8, 9, nx)
+    vol = _vol(shape, nx)
+    S_o = O.structure_tensor(vol, sigma, rho)
+    g = G.stages(vol, sigma, rho, (10.0, 10.0, 5.0), (0.0, 0.0, 1.0))
+    err = np.abs(g["S"] - S_o) / (S_o[0] + S_o[1] + S_o[2])[None]
+    assert err.max() <= 2e-5, err.max()  # the stage's tolerance (FP32 form)
+
+
+@pytest.mark.parametrize("x0,n0", [(0, 64), (1, 70), (3, 101), (5, 66), (29, 131), (40, 129), (96, 73), (104, 65)])
+@pytest.mark.parametrize("shape", [(40, 150, 169), (150, 20, 176)])
+@pytest.mark.parametrize("prec", [_lib.CT_PREC_FP32, _lib.CT_PREC_MIXED])
+def test_boxes_with_padded_rows_equal_the_whole(x0, n0, shape, prec):
+    sigma, rho = 1.0, 4.0
+    vol = _vol(shape, 5)
+    nz, ny, nx = shape
+    cen, ax = (80.0, 60.0, 10.0), (0.1, 0.1, 1.0)
+    whole = G.fused(vol, sigma, rho, cen, ax, precision=prec, raw=True)
+    h = O.radius(sigma) + O.radius(rho)
+    lo, n = (x0, 3, 5), (n0, ny - 7, nz - 9)
+    ilo = tuple(max(0, a - h) for a in lo)
+    ihi = tuple(min(d, a + b + h) for a, b, d in zip(lo, n, (nx, ny, nz)))
+    sub = vol[ilo[2]:ihi[2], ilo[1]:ihi[1], ilo[0]:ihi[0]]
+    o = [torch.empty((k,) * (k > 1) + (n[2], n[1], n[0]), device="cuda") for k in (3, 1, 1, 1)]
+    plan = _lib.ct_plan_create(_lib.make_params(sigma, rho, cen, ax, prec), (nx, ny, nz))
+    try:
+        _lib.ct_run_box(plan, G.dev_u16(sub), ilo, tuple(b - a for a, b in zip(ilo, ihi)), lo, n, None, *o)
+        torch.cuda.synchronize()
+        _lib.ct_plan_sync(plan)
+    finally:
+        _lib.ct_plan_destroy(plan)
+    sl = (slice(lo[2], lo[2] + n[2]), slice(lo[1], lo[1] + n[1]), slice(lo[0], lo[0] + n[0]))
+    for k, t in zip(("v", "ha", "ia", "fa"), o):
+        np.testing.assert_array_equal(t.cpu().numpy(), whole[k][(slice(None),) * (k == "v") + sl], err_msg=k)
