@@ -67,3 +67,29 @@ def test_boxes_with_padded_rows_equal_the_whole(x0, n0, shape, prec):
     sl = (slice(lo[2], lo[2] + n[2]), slice(lo[1], lo[1] + n[1]), slice(lo[0], lo[0] + n[0]))
     for k, t in zip(("v", "ha", "ia", "fa"), o):
         np.testing.assert_array_equal(t.cpu().numpy(), whole[k][(slice(None),) * (k == "v") + sl], err_msg=k)
+
+
+@pytest.mark.parametrize("ny,nz", [(1, 1), (31, 1), (33, 1), (32, 3), (127, 1), (129, 1), (20, 24), (25, 41)])
+def test_tensor_core_rows_of_every_count(monkeypatch, ny, nz):
+    """The tensor-core x pass takes each component's rows in groups of 128, the last one ragged
+    (tensor maps read its missing rows as zeros and clip their stores): the tensor matches the
+    oracle in every row, and nothing is written past the last component's last row."""
+    monkeypatch.setenv("CT_TUNE_TC_RHO", "7")
+    monkeypatch.setenv("CT_TUNE_TC_MIN_R", "0")
+    monkeypatch.setenv("CT_TUNE_TC_ANY_BOX", "1")
+    nx, sigma, rho = 192, 1.0, 3.0
+    vol = _vol((nz, ny, nx), 17 * ny + nz)
+    n = nx * ny * nz
+    plan = _lib.ct_plan_create(_lib.make_params(sigma, rho, (0, 0, 0), (0, 0, 1)), (nx, ny, nz))
+    try:
+        S = torch.full((6 * n + 4096,), -7.0, device="cuda")
+        _lib.ct_structure_tensor(plan, G.dev_u16(vol), (0, 0, 0), (nx, ny, nz), (0, 0, 0), (nx, ny, nz), S)
+        torch.cuda.synchronize()
+        _lib.ct_plan_sync(plan)
+    finally:
+        _lib.ct_plan_destroy(plan)
+    S = S.cpu().numpy()
+    assert np.all(S[6 * n:] == -7.0)
+    S_o = O.structure_tensor(vol, sigma, rho)
+    err = np.abs(S[:6 * n].reshape(S_o.shape) - S_o) / (S_o[0] + S_o[1] + S_o[2])[None]
+    assert err.max() <= 2e-5, err.max()
