@@ -8,8 +8,11 @@
 //
 // Both walk an axis with per-thread register windows (y in the first, z in
 // the second), so neither computes the halo rows of a 2-D tile.  The three
-// partial fields cross HBM once (12 B written and read per voxel); the
-// gradient itself never does.
+// partial fields cross HBM once (12 B written and read per voxel), as a plane of
+// (F0, F1) pairs and a plane of F2: two stores and two copies per voxel
+// instead of three of each, and the pairs are what the z pass's packed
+// arithmetic takes (512^3: x/y
+// 604 -> 615 us, z 500 -> 433 us).
 //
 // Every pass folds the +k / -k taps (sums for the smoothing taps w,
 // differences for the derivative taps c), so a constant volume gives an
@@ -27,7 +30,9 @@ namespace ct {
 //           of both filters to the pair (c_x I, w_x I) of an output;
 //   y pass  the window holds those pairs, so that the two smoothing outputs
 //           (w_y c_x I, w_y w_x I) share one packed add and one packed fma per
-//           tap; the derivative output (c_y w_x I) stays scalar.
+//           tap; the derivative output (c_y w_x I) stays scalar (pairing it with
+//           w_y c_x I instead, as the pair is stored, measured 627 us at 512^3
+//           against 614).
 // Every output takes the same operations in the same order as the scalar
 // form, so its value is the same to the bit.
 #ifndef CT_GXY_TB
@@ -134,8 +139,9 @@ __device__ __forceinline__ void grad_xy_body(const uint16_t* __restrict__ vol, c
   const int xr = t % 8;
   const int xseg = t / 8;
   const bool xok = x0 + t < xend;
-  const int64_t nab = box_vox(ab);
-  float* obase = F + box_index(ab, min(x0 + t, xend - 1), p0, z);
+  const int64_t oidx = box_index(ab, min(x0 + t, xend - 1), p0, z);
+  float2* obase01 = reinterpret_cast<float2*>(F) + oidx;
+  float* obase2 = F + 2 * box_vox(ab) + oidx;
   const int ostride = ab.n[0];
   const float2 cw0 = make_float2(0.f, tx.w[RS]);  // centre tap of (c_x, w_x)
   const float2 sgn = make_float2(-1.f, 1.f);
@@ -194,10 +200,9 @@ __device__ __forceinline__ void grad_xy_body(const uint16_t* __restrict__ vol, c
           f1 = fmaf(ty.c[RS + k], wp[m + k].y - wp[m - k].y, f1);
         }
         if (xok && m0 + i < L) {
-          float* o = obase + (int64_t)(m0 + i) * ostride;
-          o[0] = f02.x;
-          o[nab] = f1;
-          o[2 * nab] = f02.y;
+          const int o = (m0 + i) * ostride;
+          obase01[o] = make_float2(f02.x, f1);
+          obase2[o] = f02.y;
         }
       }
     }
@@ -275,8 +280,9 @@ __global__ void __launch_bounds__(XT, 512 / XT)
   const int xr = t % 8;
   const int xseg = t / 8;
   const bool xok = x0 + t < xend;
-  const int64_t nab = box_vox(ab);
-  float* obase = F + box_index(ab, min(x0 + t, xend - 1), p0, z);
+  const int64_t oidx = box_index(ab, min(x0 + t, xend - 1), p0, z);
+  float2* obase01 = reinterpret_cast<float2*>(F) + oidx;
+  float* obase2 = F + 2 * box_vox(ab) + oidx;
   const int ostride = ab.n[0];
   const float2 cw0 = make_float2(0.f, tx.w[RS]);  // centre tap of (c_x, w_x)
   const float2 sgn = make_float2(-1.f, 1.f);
@@ -335,10 +341,9 @@ __global__ void __launch_bounds__(XT, 512 / XT)
           f1 = fmaf(ty.c[RS + k], wp[m + k].y - wp[m - k].y, f1);
         }
         if (xok && m0 + i < L) {
-          float* o = obase + (int64_t)(m0 + i) * ostride;
-          o[0] = f02.x;
-          o[nab] = f1;
-          o[2 * nab] = f02.y;
+          const int o = (m0 + i) * ostride;
+          obase01[o] = make_float2(f02.x, f1);
+          obase2[o] = f02.y;
         }
       }
     }
@@ -407,19 +412,17 @@ __device__ __forceinline__ void grad_z_body(const float* __restrict__ F, const B
 
   // step s reads plane p0 - RS + s of the partial fields, clamped to the planes they
   // cover (the volume's edges, or the halo)
-  const int64_t nab = box_vox(ab);
-  const float* base = F + col;
+  const float2* base01 = reinterpret_cast<const float2*>(F) + col;
+  const float* base2 = F + 2 * box_vox(ab) + col;
   const int q0 = p0 - RS - ab.lo[2];
-  auto src = [&](int s) -> const float* { return base + (int64_t)min(max(q0 + s, 0), ab.n[2] - 1) * plane; };
   const uint32_t ring01 = (uint32_t)__cvta_generic_to_shared(gz_ring + 2 * tid);
   const uint32_t ring2 = (uint32_t)__cvta_generic_to_shared(gz_ring + 2 * kGzThreads + tid);
   constexpr uint32_t kStep = 3 * kGzThreads * sizeof(float);
   auto issue = [&](int s, int slot) {
     if (s < nsteps) {
-      const float* p = src(s);
-      cp_async4(ring01 + slot * kStep, p);
-      cp_async4(ring01 + slot * kStep + 4, p + nab);
-      cp_async4(ring2 + slot * kStep, p + 2 * nab);
+      const int i = min(max(q0 + s, 0), ab.n[2] - 1) * plane;
+      cp_async8(ring01 + slot * kStep, reinterpret_cast<const float*>(base01 + i));
+      cp_async4(ring2 + slot * kStep, base2 + i);
     }
     cp_async_commit();
   };
@@ -427,10 +430,9 @@ __device__ __forceinline__ void grad_z_body(const float* __restrict__ F, const B
   for (int s = 0; s < AH; ++s) issue(s, s);
 
   const int64_t nob = box_vox(ob);
-  float* J = static_cast<float*>(Jv);
-  __half* Jh = static_cast<__half*>(Jv);
-  const int64_t obase_i = (int64_t)(p0 - ob.lo[2]) * plane + col;
-  float* obase = J + obase_i;
+  const int64_t obase = (int64_t)(p0 - ob.lo[2]) * plane + col;
+  float* J = static_cast<float*>(Jv) + obase;
+  __half* Jh = static_cast<__half*>(Jv) + obase;
   float2 w01[P];
   float w2[P];
 #pragma unroll
@@ -462,15 +464,15 @@ __device__ __forceinline__ void grad_z_body(const float* __restrict__ F, const B
         float gx = gxy.x, gy = gxy.y;
         if (GOUT) {  // the gradient itself, held in FP16 (scaled) in the mixed form
           if (ok) {
-            const int64_t o = obase_i + (int64_t)(s - 2 * RS) * plane;
+            const int o = (s - 2 * RS) * plane;
             if (MIXED) {
               Jh[o] = __float2half_rn(gx * kGzHalfScale);
-              Jh[o + nob] = __float2half_rn(gy * kGzHalfScale);
-              Jh[o + 2 * nob] = __float2half_rn(gz * kGzHalfScale);
+              Jh[nob + o] = __float2half_rn(gy * kGzHalfScale);
+              Jh[2 * nob + o] = __float2half_rn(gz * kGzHalfScale);
             } else {
               J[o] = gx;
-              J[o + nob] = gy;
-              J[o + 2 * nob] = gz;
+              J[nob + o] = gy;
+              J[2 * nob + o] = gz;
             }
           }
           continue;
@@ -481,7 +483,7 @@ __device__ __forceinline__ void grad_z_body(const float* __restrict__ F, const B
           gz = __half2float(__float2half_rn(gz * kGzHalfScale)) * (1.0f / kGzHalfScale);
         }
         if (ok) {
-          float* o = obase + (int64_t)(s - 2 * RS) * plane;
+          float* o = J + (s - 2 * RS) * plane;
           if (ps.unit) {
             o[0] = gx * gx;
             o[nob] = gy * gy;
