@@ -80,7 +80,9 @@ __device__ __forceinline__ void rho_xy_body(const float* __restrict__ in, const 
   // This thread's 16-byte chunks of a staged block: chunk q = t + kXT i is row
   // q / QW, columns 4 (q % QW) .. +3.  Column-dependent parts are fixed for the
   // walk; a chunk is copied by cp.async when it lies inside the input box and
-  // rows are 16-byte aligned, else element by element with clamping.
+  // rows are 16-byte aligned, else element by element with clamping (asynchronous
+  // too: loads waited for here would hold up every block of a CTA at the
+  // volume's edge).
   constexpr int NQ = (kTB * G::QW + kXT - 1) / kXT;
   int q_row[NQ], q_col[NQ];
   bool q_fast[NQ];
@@ -105,12 +107,10 @@ __device__ __forceinline__ void rho_xy_body(const float* __restrict__ in, const 
       if (q_fast[i]) {
         cp_async16(stage0 + (uint32_t)so * 4u, row + q_col[i]);
       } else {
-        float* d = stage + so;
+        const uint32_t d = stage0 + (uint32_t)so * 4u;
         const int gx0 = q_col[i];
-        d[0] = __ldg(row + clamp_to(gx0, dimx, ib.lo[0], ib.n[0]));
-        d[1] = __ldg(row + clamp_to(gx0 + 1, dimx, ib.lo[0], ib.n[0]));
-        d[2] = __ldg(row + clamp_to(gx0 + 2, dimx, ib.lo[0], ib.n[0]));
-        d[3] = __ldg(row + clamp_to(gx0 + 3, dimx, ib.lo[0], ib.n[0]));
+#pragma unroll
+        for (int e = 0; e < 4; ++e) cp_async4(d + 4 * e, row + clamp_to(gx0 + e, dimx, ib.lo[0], ib.n[0]));
       }
     }
   };
@@ -241,7 +241,9 @@ __global__ void __launch_bounds__(XT, CT_XY_MINB * 256 / XT)
   // This thread's 16-byte chunks of a staged block: chunk q = t + kXT i is row
   // q / QW, columns 4 (q % QW) .. +3.  Column-dependent parts are fixed for the
   // walk; a chunk is copied by cp.async when it lies inside the input box and
-  // rows are 16-byte aligned, else element by element with clamping.
+  // rows are 16-byte aligned, else element by element with clamping (asynchronous
+  // too: loads waited for here would hold up every block of a CTA at the
+  // volume's edge).
   constexpr int NQ = (kTB * G::QW + kXT - 1) / kXT;
   int q_row[NQ], q_col[NQ];
   bool q_fast[NQ];
@@ -266,12 +268,10 @@ __global__ void __launch_bounds__(XT, CT_XY_MINB * 256 / XT)
       if (q_fast[i]) {
         cp_async16(stage0 + (uint32_t)so * 4u, row + q_col[i]);
       } else {
-        float* d = stage + so;
+        const uint32_t d = stage0 + (uint32_t)so * 4u;
         const int gx0 = q_col[i];
-        d[0] = __ldg(row + clamp_to(gx0, dimx, ib.lo[0], ib.n[0]));
-        d[1] = __ldg(row + clamp_to(gx0 + 1, dimx, ib.lo[0], ib.n[0]));
-        d[2] = __ldg(row + clamp_to(gx0 + 2, dimx, ib.lo[0], ib.n[0]));
-        d[3] = __ldg(row + clamp_to(gx0 + 3, dimx, ib.lo[0], ib.n[0]));
+#pragma unroll
+        for (int e = 0; e < 4; ++e) cp_async4(d + 4 * e, row + clamp_to(gx0 + e, dimx, ib.lo[0], ib.n[0]));
       }
     }
   };

@@ -4,6 +4,9 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
+#include <cmath>
+
 #include "ct_common.cuh"
 
 namespace ct {
@@ -17,9 +20,9 @@ cudaError_t prepare_grad_split_kernels();
 // walk n positions each, a segment of L of them costing L + warm (warm: the
 // steps before its first output, in steps of the walk), and `slots` CTAs are
 // resident at once on `sms` SMs.  The cheapest of up to 64 cuts, whole waves
-// of CTAs counted as they run side by side, the last one by the CTAs per SM it
-// still holds but no less than kLoneCta of a full wave (a lone CTA waits for
-// its own loads and barriers).  seg: a multiple of unit.  Before, the walks were
+// of CTAs counted as they run side by side, the last one by the square root of
+// the share of an SM's CTAs it still holds (fewer CTAs run faster, but not in
+// proportion) and no less than kLoneCta (one waits for its own loads and barriers).  seg: a multiple of unit.  Before, the walks were
 // cut by powers of two while the grid was below a fixed size and a segment
 // above a fixed length, so a 64^3 volume ran grad_z in 16 CTAs: its gradient
 // x/y, z and rho z passes 15.4, 16.4, 10.4 us, and 10.8, 8.3, 8.1 now;
@@ -36,8 +39,8 @@ inline int walk_segment(int64_t ctas, int n, int unit, double warm, int slots, i
     const int64_t full = total / slots, rest = total - full * slots;
     double waves = (double)full;
     if (rest) {
-      const double r = (double)((rest + sms - 1) / sms) * sms / slots;
-      waves += r > kLoneCta ? (r < 1.0 ? r : 1.0) : kLoneCta;
+      const double r = std::sqrt(std::min(1.0, (double)((rest + sms - 1) / sms) * sms / slots));
+      waves += std::max(r, kLoneCta);
     }
     const double cost = waves * (seg + warm);
     if (cost < best * 0.99) best = cost, best_seg = seg;  // a finer cut only where it gains
