@@ -348,22 +348,27 @@ __device__ __noinline__ void eig_jacobi(const Sym3<T>& s, T l[3], T v[3]) {
   for (int sweep = 0; sweep < 32; ++sweep) {
     T off = sqrt(T(2) * (A[0][1] * A[0][1] + A[0][2] * A[0][2] + A[1][2] * A[1][2]));
     if (off <= tol || off == T(0)) break;
+#pragma unroll
     for (int p = 0; p < 2; ++p) {
+#pragma unroll
       for (int qq = p + 1; qq < 3; ++qq) {
         if (A[p][qq] == T(0)) continue;
         T tau = (A[qq][qq] - A[p][p]) / (T(2) * A[p][qq]);
         T t = (tau >= T(0) ? T(1) : T(-1)) / (fabs(tau) + sqrt(T(1) + tau * tau));
         T cs = T(1) / sqrt(T(1) + t * t), sn = t * cs;
+#pragma unroll
         for (int k = 0; k < 3; ++k) {
           T akp = A[k][p], akq = A[k][qq];
           A[k][p] = cs * akp - sn * akq;
           A[k][qq] = sn * akp + cs * akq;
         }
+#pragma unroll
         for (int k = 0; k < 3; ++k) {
           T apk = A[p][k], aqk = A[qq][k];
           A[p][k] = cs * apk - sn * aqk;
           A[qq][k] = sn * apk + cs * aqk;
         }
+#pragma unroll
         for (int k = 0; k < 3; ++k) {
           T qkp = Q[k][p], qkq = Q[k][qq];
           Q[k][p] = cs * qkp - sn * qkq;
@@ -372,14 +377,23 @@ __device__ __noinline__ void eig_jacobi(const Sym3<T>& s, T l[3], T v[3]) {
       }
     }
   }
+  // ascending, the smallest one's vector carried along (no indexed access: the
+  // matrices stay in registers)
   T d0 = A[0][0], d1 = A[1][1], d2 = A[2][2];
-  int i0 = 0, i1 = 1, i2 = 2;
-  if (d1 < d0) { T t = d0; d0 = d1; d1 = t; int u = i0; i0 = i1; i1 = u; }
-  if (d2 < d1) { T t = d1; d1 = d2; d2 = t; int u = i1; i1 = i2; i2 = u; }
-  if (d1 < d0) { T t = d0; d0 = d1; d1 = t; int u = i0; i0 = i1; i1 = u; }
+  T v0[3] = {Q[0][0], Q[1][0], Q[2][0]}, v1[3] = {Q[0][1], Q[1][1], Q[2][1]};
+  const T v2[3] = {Q[0][2], Q[1][2], Q[2][2]};
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const bool s01 = d1 < d0;
+    const T lo = s01 ? v1[k] : v0[k], hi = s01 ? v0[k] : v1[k];
+    const T m0 = s01 ? d1 : d0, m1 = s01 ? d0 : d1;
+    const T mid = d2 < m1 ? v2[k] : hi, dm = d2 < m1 ? d2 : m1;
+    v[k] = dm < m0 ? mid : lo;
+  }
+  if (d1 < d0) { T t = d0; d0 = d1; d1 = t; }
+  if (d2 < d1) { T t = d1; d1 = d2; d2 = t; }
+  if (d1 < d0) { T t = d0; d0 = d1; d1 = t; }
   l[0] = d0; l[1] = d1; l[2] = d2;
-  v[0] = Q[0][i0]; v[1] = Q[1][i0]; v[2] = Q[2][i0];
-  (void)i2;
 }
 
 // Fractional anisotropy from eigenvalues clamped at zero; 0 for the zero tensor.
