@@ -195,6 +195,7 @@ struct ct_plan_s {
   uint64_t graph_key = 0;
   int64_t graph_launches = 0, graph_voxels = 0;
   bool capturing = false;
+  uint64_t ready_s = 0, ready_r = 0;  // radii whose kernels' attributes are set (ensure_kernels)
   ct_stats stats;
   std::mutex mu;
   int stream_block = 16;  // outputs per thread block of the y / z passes (tuning choice)
@@ -282,6 +283,21 @@ ct_status make_scale(const ct_params& p, double sigma, double rho, Scale* s) {
   }
   static const int ca[6] = {0, 1, 2, 0, 0, 1}, cb[6] = {0, 1, 2, 1, 2, 2};
   for (int k = 0; k < 6; ++k) s->ss[k] = (float)(1.0 / (sp[ca[k]] * sp[cb[k]]));
+  return CT_OK;
+}
+
+// The attributes of the kernels of this scale's radii, once per plan: a plan
+// uses few of the instantiations (all of them took 0.8 ms per plan).
+ct_status ensure_kernels(ct_plan P, const Scale& sc) {
+  if (!(P->ready_s >> sc.rks & 1)) {
+    CT_CUDA(prepare_grad_split_kernels(sc.rks), "kernel attribute set-up");
+    P->ready_s |= uint64_t(1) << sc.rks;
+  }
+  if (!(P->ready_r >> sc.rkr & 1)) {
+    CT_CUDA(prepare_rho_xy_kernels(sc.rkr), "kernel attribute set-up");
+    CT_CUDA(prepare_rho_tc_kernels(sc.rkr), "kernel attribute set-up");
+    P->ready_r |= uint64_t(1) << sc.rkr;
+  }
   return CT_OK;
 }
 
@@ -488,11 +504,16 @@ ChainBoxes chain_boxes(const Scale& sc, const int dims[3], const Box& vb, const 
   return c;
 }
 
+Queue queue_of(ct_plan P, const Box& ob, cudaStream_t st) {
+  return Queue(st, box_vox(ob) <= kEarlyMaxVox && !P->capturing);
+}
+
 ct_status smooth_chain(ct_plan P, const Scale& sc, const int dims[3], const uint16_t* vol, const Box& vb,
-                       const Box& ob, int slot, bool mixed, cudaStream_t st, float* S_out, float** S_res,
+                       const Box& ob, int slot, bool mixed, cudaStream_t st, int* zero, float* S_out, float** S_res,
                        Box* S_box) {
   const ChainBoxes cb = chain_boxes(sc, dims, vb, ob);
   const Box &G = cb.G, &Ab = cb.Ab;
+  const Queue q = queue_of(P, ob, st);
   const Box So = S_out ? ob : cb.S;  // a caller's tensor is dense
   *S_box = So;
   ct_status rc = ensure_scratch(P, slot, cb.need);
@@ -502,7 +523,7 @@ ct_status smooth_chain(ct_plan P, const Scale& sc, const int dims[3], const uint
   const auto* tuning = tuned(P, sc, dims);
   const TcCtl ctl{P->d_timeouts, P->tc_wait_limit, tuning ? tuning->seg_cap : 0};
   const int sblock = tuning && tuning->stream_block ? tuning->stream_block : P->stream_block;
-  CT_LAUNCH(P, st, "grad_xy", launch_grad_xy(vol, vb, dims, B, Ab, sc.ts[0], sc.ts[1], sc.rks, st),
+  CT_LAUNCH(P, st, "grad_xy", launch_grad_xy(vol, vb, dims, B, Ab, sc.ts[0], sc.ts[1], sc.rks, zero, q),
             "gradient x/y kernel launch");
   const bool tcx = use_tc(P, sc, dims, 0), tcy = use_tc(P, sc, dims, 1), tcz = use_tc(P, sc, dims, 2);
   if (tcx && tcy && tcz && (tuning ? tuning->rho_path == 2 : P->tc_products)) {
@@ -513,13 +534,13 @@ ct_status smooth_chain(ct_plan P, const Scale& sc, const int dims[3], const uint
     Bzy.n[1] = ob.n[1];
     float* S = S_out ? S_out : B;
     CT_LAUNCH(P, st, mixed ? "grad_z_g16" : "grad_z_g32",
-              launch_grad_z(B, Ab, A, G, sc.ts[2], sc.ss, sc.rks, mixed, true, st), "gradient z kernel launch");
+              launch_grad_z(B, Ab, A, G, sc.ts[2], sc.ss, sc.rks, mixed, true, q), "gradient z kernel launch");
     CT_LAUNCH(P, st, mixed ? "rho_z_tc_g16" : "rho_z_tc_g32",
-              launch_rho_tc_products(A, mixed, G, dims, B, Bz, 2, sc.tr[2], sc.ss, sc.rkr, ctl, st),
+              launch_rho_tc_products(A, mixed, G, dims, B, Bz, 2, sc.tr[2], sc.ss, sc.rkr, ctl, q),
               "rho z kernel launch");
-    CT_LAUNCH(P, st, "rho_y_tc", launch_rho_tc(B, Bz, dims, A, Bzy, 1, sc.tr[1], sc.rkr, ctl, st),
+    CT_LAUNCH(P, st, "rho_y_tc", launch_rho_tc(B, Bz, dims, A, Bzy, 1, sc.tr[1], sc.rkr, ctl, q),
               "rho y kernel launch");
-    CT_LAUNCH(P, st, "rho_x_tc", launch_rho_tc(A, Bzy, dims, S, So, 0, sc.tr[0], sc.rkr, ctl, st),
+    CT_LAUNCH(P, st, "rho_x_tc", launch_rho_tc(A, Bzy, dims, S, So, 0, sc.tr[0], sc.rkr, ctl, q),
               "rho x kernel launch");
     *S_res = S;
     return CT_OK;
@@ -529,7 +550,7 @@ ct_status smooth_chain(ct_plan P, const Scale& sc, const int dims[3], const uint
   Bx.n[0] = Bxy.n[0] = cb.S.n[0];
   Bxy.lo[1] = ob.lo[1];
   Bxy.n[1] = ob.n[1];
-  CT_LAUNCH(P, st, "grad_z", launch_grad_z(B, Ab, A, G, sc.ts[2], sc.ss, sc.rks, mixed, false, st),
+  CT_LAUNCH(P, st, "grad_z", launch_grad_z(B, Ab, A, G, sc.ts[2], sc.ss, sc.rks, mixed, false, q),
             "gradient z kernel launch");
   // x and y on the tensor cores together, or as one fused FP32 stencil; a mask
   // that selects one of the two axes (tuning, tests) runs them as separate passes
@@ -537,27 +558,27 @@ ct_status smooth_chain(ct_plan P, const Scale& sc, const int dims[3], const uint
   float* Sxy;
   if ((tcx && tcy) || (one_axis && (tcx || tcy))) {
     if (tcx)
-      CT_LAUNCH(P, st, "rho_x_tc", launch_rho_tc(A, G, dims, B, Bx, 0, sc.tr[0], sc.rkr, ctl, st),
+      CT_LAUNCH(P, st, "rho_x_tc", launch_rho_tc(A, G, dims, B, Bx, 0, sc.tr[0], sc.rkr, ctl, q),
                 "rho x kernel launch");
     else
-      CT_LAUNCH(P, st, "rho_x", launch_rho_x(A, G, dims, B, Bx, sc.tr[0], sc.rkr, st), "rho x kernel launch");
+      CT_LAUNCH(P, st, "rho_x", launch_rho_x(A, G, dims, B, Bx, sc.tr[0], sc.rkr, q), "rho x kernel launch");
     if (tcy)
-      CT_LAUNCH(P, st, "rho_y_tc", launch_rho_tc(B, Bx, dims, A, Bxy, 1, sc.tr[1], sc.rkr, ctl, st),
+      CT_LAUNCH(P, st, "rho_y_tc", launch_rho_tc(B, Bx, dims, A, Bxy, 1, sc.tr[1], sc.rkr, ctl, q),
                 "rho y kernel launch");
     else
-      CT_LAUNCH(P, st, "rho_y", launch_rho_stream(B, Bx, dims, A, Bxy, 1, sc.tr[1], sc.rkr, sblock, st),
+      CT_LAUNCH(P, st, "rho_y", launch_rho_stream(B, Bx, dims, A, Bxy, 1, sc.tr[1], sc.rkr, sblock, q),
                 "rho y kernel launch");
     Sxy = A;
   } else {
-    CT_LAUNCH(P, st, "rho_xy", launch_rho_xy(A, G, dims, B, Bxy, sc.tr[0], sc.tr[1], sc.rkr, st), "rho xy kernel launch");
+    CT_LAUNCH(P, st, "rho_xy", launch_rho_xy(A, G, dims, B, Bxy, sc.tr[0], sc.tr[1], sc.rkr, q), "rho xy kernel launch");
     Sxy = B;
   }
   float* S = S_out ? S_out : (Sxy == A ? B : A);
   if (tcz)
-    CT_LAUNCH(P, st, "rho_z_tc", launch_rho_tc(Sxy, Bxy, dims, S, So, 2, sc.tr[2], sc.rkr, ctl, st),
+    CT_LAUNCH(P, st, "rho_z_tc", launch_rho_tc(Sxy, Bxy, dims, S, So, 2, sc.tr[2], sc.rkr, ctl, q),
               "rho z kernel launch");
   else
-    CT_LAUNCH(P, st, "rho_z", launch_rho_stream(Sxy, Bxy, dims, S, So, 2, sc.tr[2], sc.rkr, sblock, st),
+    CT_LAUNCH(P, st, "rho_z", launch_rho_stream(Sxy, Bxy, dims, S, So, 2, sc.tr[2], sc.rkr, sblock, q),
               "rho z kernel launch");
   *S_res = S;
   return CT_OK;
@@ -568,7 +589,7 @@ ct_status tensor_stages(ct_plan P, const Scale& sc, const int dims[3], const uin
                         const Box& ob, float* S_out, int slot, bool mixed, cudaStream_t st) {
   float* S = nullptr;
   Box sb;
-  return smooth_chain(P, sc, dims, vol, vb, ob, slot, mixed, st, S_out, &S, &sb);
+  return smooth_chain(P, sc, dims, vol, vb, ob, slot, mixed, st, nullptr, S_out, &S, &sb);
 }
 
 ct_status eig_stage(ct_plan P, const float* S, const Box& sb, const Box& ob, const uint8_t* mask, const Box& mb, const Frame& F,
@@ -582,7 +603,11 @@ ct_status fused_stages(ct_plan P, const Scale& sc, const int dims[3], const uint
                        bool mixed, cudaStream_t st) {
   float* S = nullptr;
   Box sb;
-  ct_status rc = smooth_chain(P, sc, dims, vol, vb, ob, slot, mixed, st, nullptr, &S, &sb);
+  ct_status rc = ensure_fallback(P, slot, box_vox(ob));
+  // the chain's first kernel clears the re-solve counter (a memset between the
+  // kernels would keep the next one from starting early)
+  if (rc == CT_OK)
+    rc = smooth_chain(P, sc, dims, vol, vb, ob, slot, mixed, st, P->fb_count[slot], nullptr, &S, &sb);
   if (rc) return rc;
   const auto* t = tuned(P, sc, dims);
   return eig_stage(P, S, sb, ob, mask, mb, F, o, slot, mixed, t && t->eig_compact >= 0 ? t->eig_compact != 0 : P->eig_compact,
@@ -592,13 +617,13 @@ ct_status fused_stages(ct_plan P, const Scale& sc, const int dims[3], const uint
 // Eigen + angles over ob from S (over sb); outputs in arrays covering o.ab.
 ct_status eig_stage(ct_plan P, const float* S, const Box& sb, const Box& ob, const uint8_t* mask, const Box& mb, const Frame& F,
                     const EigOut& o, int slot, bool mixed, bool compact, cudaStream_t st) {
-  Fallback fb = fallback_of(P, slot);
-  CT_CUDA(cudaMemsetAsync(fb.count, 0, sizeof(int), st), "counter reset");
+  const Queue q = queue_of(P, ob, st);
+  Fallback fb = fallback_of(P, slot);  // its counter was cleared by the chain
   CT_LAUNCH(P, st, "eig_angles",
-            launch_eig_angles(S, sb, ob, mask, mb, F, P->p.fill_value, o, mixed, fb, compact, st),
+            launch_eig_angles(S, sb, ob, mask, mb, F, P->p.fill_value, o, mixed, fb, compact, q),
             "eigen kernel launch");
   CT_LAUNCH(P, st, "eig_resolve",
-            launch_eig_angles_fallback(S, sb, ob, mask, mb, F, P->p.fill_value, o, mixed, fb, box_vox(ob), st),
+            launch_eig_angles_fallback(S, sb, ob, mask, mb, F, P->p.fill_value, o, mixed, fb, box_vox(ob), q),
             "re-solve kernel launch");
   return CT_OK;
 }
@@ -728,12 +753,6 @@ ct_status ct_plan_create(const ct_params* params, const int64_t vol_dims[3], ct_
   Scale sc;
   if ((rc = make_scale(*params, params->sigma, params->rho, &sc))) return rc;
   if (!device_present()) return fail(CT_ERR_NO_DEVICE, "no CUDA device is available");
-  {
-    cudaError_t e = prepare_rho_xy_kernels();
-    if (e == cudaSuccess) e = prepare_grad_split_kernels();
-    if (e == cudaSuccess) e = prepare_rho_tc_kernels();
-    if (e != cudaSuccess) return cuda_fail(e, "kernel attribute set-up");
-  }
   ct_plan P = new (std::nothrow) ct_plan_s();
   if (!P) return fail(CT_ERR_OOM, "plan allocation failed");
   P->p = *params;
@@ -758,6 +777,10 @@ ct_status ct_plan_create(const ct_params* params, const int64_t vol_dims[3], ct_
     }
   }
   std::memset(&P->stats, 0, sizeof P->stats);
+  if ((rc = ensure_kernels(P, sc))) {
+    ct_plan_destroy(P);
+    return rc;
+  }
   if (const char* e = std::getenv("CT_TUNE_STREAM_BLOCK")) P->stream_block = std::atoi(e) == 8 ? 8 : 16;
   if (const char* e = std::getenv("CT_TUNE_TC_RHO")) P->tc_rho = std::atoi(e) & 7;
   if (const char* e = std::getenv("CT_TUNE_TC_ANY_BOX")) P->tc_any_box = std::atoi(e) != 0;
@@ -875,7 +898,7 @@ ct_status ct_eig_smallest(ct_plan P, const float* d_S, int64_t n, float* d_evals
   bool mixed = P->p.precision == CT_PREC_MIXED;
   CT_CUDA(cudaMemsetAsync(fb.count, 0, sizeof(int), st), "counter reset");
   CT_LAUNCH(P, st, "eig_only", launch_eig_only(d_S, n, d_evals, d_evec, mixed, fb, st), "eigen kernel launch");
-  CT_LAUNCH(P, st, "eig_only_resolve", launch_eig_only_fallback(d_S, n, d_evals, d_evec, mixed, fb, n, st),
+  CT_LAUNCH(P, st, "eig_only_resolve", launch_eig_only_fallback(d_S, n, d_evals, d_evec, mixed, fb, n, Queue(st, n <= kEarlyMaxVox)),
             "re-solve kernel launch");
   return mark(P, st);
 }
@@ -961,6 +984,7 @@ ct_status item_ctx(ct_plan P, const ct_item& it, ItemCtx* c) {
   double sig = it.sigma > 0.0 ? it.sigma : P->p.sigma;
   double rho = it.rho > 0.0 ? it.rho : P->p.rho;
   ct_status rc = make_scale(P->p, sig, rho, &c->sc);
+  if (rc == CT_OK) rc = ensure_kernels(P, c->sc);
   if (rc) return rc;
   bool own_axis = it.lv_axis[0] != 0.0 || it.lv_axis[1] != 0.0 || it.lv_axis[2] != 0.0;
   for (int k = 0; k < 3; ++k)

@@ -48,6 +48,15 @@ __device__ __forceinline__ int clamp_to(int p, int dim, int lo, int n) {
   return clampi(clampi(p, 0, dim - 1), lo, lo + n - 1);
 }
 
+// First statement of the chain's kernels, which are launched so that their CTAs
+// may start while the previous kernel of the stream still runs (launch_after):
+// waits until that kernel has finished and its writes are visible, then lets
+// the next kernel's CTAs start.  Nothing of the kernel's work comes before it.
+__device__ __forceinline__ void after_previous() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // ---------------------------------------------------------------------------
 // Persistent multi-item launches.  A stage kernel's body reads its block index
 // and grid size from a VBlock instead of blockIdx / gridDim: the single-item
@@ -117,10 +126,6 @@ __device__ __forceinline__ void for_each_vblock(const MultiTable& T, F&& f) {
     }
   }
 }
-
-// The CTA's barrier, for kernels whose warps reach it from different loops (every
-// warp as often; __syncthreads() wants one place for all).
-__device__ __forceinline__ void cta_barrier() { asm volatile("bar.sync 0;" ::: "memory"); }
 
 // Asynchronous 4- and 8-byte global -> shared copies (cp.async), grouped per commit.
 __device__ __forceinline__ void cp_async4(uint32_t smem_dst, const float* gsrc) {

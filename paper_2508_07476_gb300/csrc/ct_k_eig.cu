@@ -96,6 +96,7 @@ template <int VT, int AT, int FT>
 __global__ void __launch_bounds__(256, CT_EIG_MINB)
     k_eig_angles(const float* __restrict__ S, Box sb, Box ob, const uint8_t* __restrict__ mask, Box mb, Frame F,
                  float fill, EigOut o, bool mixed, Fallback fb) {
+  after_previous();
   const int x = ob.lo[0] + blockIdx.x * blockDim.x + threadIdx.x;
   if (x >= ob.lo[0] + ob.n[0]) return;
   const int row = blockIdx.z * gridDim.y + blockIdx.y;  // y + ny * z within ob
@@ -147,6 +148,7 @@ __global__ void __launch_bounds__(256, CT_EIG_MINB)
     k_eig_angles32(const float* __restrict__ S, Box sb, Box ob, const uint8_t* __restrict__ mask, Box mb, Frame F,
                    float fill, EigOut o, bool mixed, Fallback fb) {
   (void)mixed;
+  after_previous();
   eig32_body<VT, AT, FT, PLAIN>(S, sb, ob, mask, mb, F, fill, o, fb, HwBlock{});
 }
 
@@ -253,6 +255,7 @@ __global__ void __launch_bounds__(kEigThreads, CT_EIG_MINB * 256 / kEigThreads)
     k_eig_angles_compact(const float* __restrict__ S, Box sb, Box ob, const uint8_t* __restrict__ mask, Box mb,
                          Frame F, float fill, EigOut o, bool mixed, Fallback fb) {
   (void)mixed;
+  after_previous();
   eig_compact_body<VT, AT, FT, PLAIN>(S, sb, ob, mask, mb, F, fill, o, fb, HwBlock{});
 }
 
@@ -277,6 +280,7 @@ __global__ void __launch_bounds__(COMPACT ? kEigThreads : kEigMultiThreads,
 __global__ void __launch_bounds__(128)
     k_eig_angles_fallback(const float* __restrict__ S, Box sb, Box ob, const uint8_t* __restrict__ mask, Box mb,
                           Frame F, float fill, EigOut o, bool mixed, Fallback fb) {
+  after_previous();
   const int64_t cnt = min((int64_t)*fb.count, fb.cap);
   const int64_t ns = box_vox(sb);
   for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < cnt; j += (int64_t)gridDim.x * blockDim.x) {
@@ -331,7 +335,7 @@ static int grid_for(int64_t n, int threads) {
 
 cudaError_t launch_eig_angles(const float* S, const Box& sb, const Box& ob, const uint8_t* mask, const Box& mb,
                               const Frame& F, float fill, const EigOut& o, bool mixed, const Fallback& fb,
-                              bool compact, cudaStream_t st) {
+                              bool compact, const Queue& st) {
   int64_t n = box_vox(ob);
   if (n == 0) return cudaSuccess;
   const int rows = ob.n[1] * ob.n[2];
@@ -350,56 +354,55 @@ cudaError_t launch_eig_angles(const float* S, const Box& sb, const Box& ob, cons
       dim3 gc((ob.n[0] + kEigSpan - 1) / kEigSpan, ob.n[1], ob.n[2]);
       if (o.vec_t == CT_OUT_F32 && o.ang_t == CT_OUT_F32 && o.fa_t == CT_OUT_F32) {
         if (plain)
-          k_eig_angles_compact<0, 0, 0, true><<<gc, kEigThreads, 0, st>>>(S, sb, ob, mask, mb, F, fill, o, mixed, fb);
+          return launch_after(k_eig_angles_compact<0, 0, 0, true>, gc, kEigThreads, 0, st, S, sb, ob, mask, mb, F, fill, o, mixed, fb);
         else
-          k_eig_angles_compact<0, 0, 0, false><<<gc, kEigThreads, 0, st>>>(S, sb, ob, mask, mb, F, fill, o, mixed, fb);
+          return launch_after(k_eig_angles_compact<0, 0, 0, false>, gc, kEigThreads, 0, st, S, sb, ob, mask, mb, F, fill, o, mixed, fb);
       } else if (o.vec_t == CT_OUT_F16 && o.ang_t == CT_OUT_F16 && o.fa_t == CT_OUT_F16) {
         if (plain)
-          k_eig_angles_compact<1, 1, 1, true><<<gc, kEigThreads, 0, st>>>(S, sb, ob, mask, mb, F, fill, o, mixed, fb);
+          return launch_after(k_eig_angles_compact<1, 1, 1, true>, gc, kEigThreads, 0, st, S, sb, ob, mask, mb, F, fill, o, mixed, fb);
         else
-          k_eig_angles_compact<1, 1, 1, false><<<gc, kEigThreads, 0, st>>>(S, sb, ob, mask, mb, F, fill, o, mixed, fb);
+          return launch_after(k_eig_angles_compact<1, 1, 1, false>, gc, kEigThreads, 0, st, S, sb, ob, mask, mb, F, fill, o, mixed, fb);
       } else if (o.ang_t == CT_OUT_U8Q && o.fa_t == CT_OUT_F16) {
-        k_eig_angles_compact<-1, 2, 1, false><<<gc, kEigThreads, 0, st>>>(S, sb, ob, mask, mb, F, fill, o, mixed, fb);
+        return launch_after(k_eig_angles_compact<-1, 2, 1, false>, gc, kEigThreads, 0, st, S, sb, ob, mask, mb, F, fill, o, mixed, fb);
       } else {
-        k_eig_angles_compact<-1, -1, -1, false><<<gc, kEigThreads, 0, st>>>(S, sb, ob, mask, mb, F, fill, o, mixed, fb);
+        return launch_after(k_eig_angles_compact<-1, -1, -1, false>, gc, kEigThreads, 0, st, S, sb, ob, mask, mb, F, fill, o, mixed, fb);
       }
-      return cudaGetLastError();
     }
     if (o.vec_t == CT_OUT_F32 && o.ang_t == CT_OUT_F32 && o.fa_t == CT_OUT_F32) {
       if (plain)
-        k_eig_angles32<0, 0, 0, true><<<g3, nt, 0, st>>>(S, sb, ob, mask, mb, F, fill, o, mixed, fb);
+        return launch_after(k_eig_angles32<0, 0, 0, true>, g3, nt, 0, st, S, sb, ob, mask, mb, F, fill, o, mixed, fb);
       else
-        k_eig_angles32<0, 0, 0, false><<<g3, nt, 0, st>>>(S, sb, ob, mask, mb, F, fill, o, mixed, fb);
+        return launch_after(k_eig_angles32<0, 0, 0, false>, g3, nt, 0, st, S, sb, ob, mask, mb, F, fill, o, mixed, fb);
     } else if (o.vec_t == CT_OUT_F16 && o.ang_t == CT_OUT_F16 && o.fa_t == CT_OUT_F16) {
       if (plain)
-        k_eig_angles32<1, 1, 1, true><<<g3, nt, 0, st>>>(S, sb, ob, mask, mb, F, fill, o, mixed, fb);
+        return launch_after(k_eig_angles32<1, 1, 1, true>, g3, nt, 0, st, S, sb, ob, mask, mb, F, fill, o, mixed, fb);
       else
-        k_eig_angles32<1, 1, 1, false><<<g3, nt, 0, st>>>(S, sb, ob, mask, mb, F, fill, o, mixed, fb);
+        return launch_after(k_eig_angles32<1, 1, 1, false>, g3, nt, 0, st, S, sb, ob, mask, mb, F, fill, o, mixed, fb);
     } else if (o.ang_t == CT_OUT_U8Q && o.fa_t == CT_OUT_F16) {
-      k_eig_angles32<-1, 2, 1, false><<<g3, nt, 0, st>>>(S, sb, ob, mask, mb, F, fill, o, mixed, fb);
+      return launch_after(k_eig_angles32<-1, 2, 1, false>, g3, nt, 0, st, S, sb, ob, mask, mb, F, fill, o, mixed, fb);
     } else {
-      k_eig_angles32<-1, -1, -1, false><<<g3, nt, 0, st>>>(S, sb, ob, mask, mb, F, fill, o, mixed, fb);
+      return launch_after(k_eig_angles32<-1, -1, -1, false>, g3, nt, 0, st, S, sb, ob, mask, mb, F, fill, o, mixed, fb);
     }
     return cudaGetLastError();
   }
   // the encodings of the common configurations are compiled in; others are read at run time
   if (o.vec_t == CT_OUT_F32 && o.ang_t == CT_OUT_F32 && o.fa_t == CT_OUT_F32)
-    k_eig_angles<0, 0, 0><<<grid, nt, 0, st>>>(S, sb, ob, mask, mb, F, fill, o, mixed, fb);
+    return launch_after(k_eig_angles<0, 0, 0>, grid, nt, 0, st, S, sb, ob, mask, mb, F, fill, o, mixed, fb);
   else if (o.vec_t == CT_OUT_F16 && o.ang_t == CT_OUT_F16 && o.fa_t == CT_OUT_F16)
-    k_eig_angles<1, 1, 1><<<grid, nt, 0, st>>>(S, sb, ob, mask, mb, F, fill, o, mixed, fb);
+    return launch_after(k_eig_angles<1, 1, 1>, grid, nt, 0, st, S, sb, ob, mask, mb, F, fill, o, mixed, fb);
   else if (o.ang_t == CT_OUT_U8Q && o.fa_t == CT_OUT_F16)
-    k_eig_angles<-1, 2, 1><<<grid, nt, 0, st>>>(S, sb, ob, mask, mb, F, fill, o, mixed, fb);
+    return launch_after(k_eig_angles<-1, 2, 1>, grid, nt, 0, st, S, sb, ob, mask, mb, F, fill, o, mixed, fb);
   else
-    k_eig_angles<-1, -1, -1><<<grid, nt, 0, st>>>(S, sb, ob, mask, mb, F, fill, o, mixed, fb);
+    return launch_after(k_eig_angles<-1, -1, -1>, grid, nt, 0, st, S, sb, ob, mask, mb, F, fill, o, mixed, fb);
   return cudaGetLastError();
 }
 
 cudaError_t launch_eig_angles_fallback(const float* S, const Box& sb, const Box& ob, const uint8_t* mask,
                                        const Box& mb, const Frame& F, float fill, const EigOut& o, bool mixed,
-                                       const Fallback& fb, int64_t max_items, cudaStream_t st) {
+                                       const Fallback& fb, int64_t max_items, const Queue& st) {
   if (max_items <= 0) return cudaSuccess;
-  k_eig_angles_fallback<<<fallback_grid(max_items), 128, 0, st>>>(S, sb, ob, mask, mb, F, fill, o, mixed, fb);
-  return cudaGetLastError();
+  return launch_after(k_eig_angles_fallback, fallback_grid(max_items), 128, 0, st, S, sb, ob, mask, mb, F, fill, o, mixed,
+                      fb);
 }
 
 // ------------------------------------------------------------ batches
@@ -509,6 +512,7 @@ __global__ void __launch_bounds__(kEigOnlyThreads)
 __global__ void __launch_bounds__(128)
     k_eig_only_fallback(const float* __restrict__ S, int64_t n, float* __restrict__ evals, float* __restrict__ evec,
                         bool mixed, Fallback fb) {
+  after_previous();
   const int64_t cnt = min((int64_t)*fb.count, fb.cap);
   for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < cnt; j += (int64_t)gridDim.x * blockDim.x) {
     const int64_t i = fb.list[j];
@@ -648,10 +652,9 @@ cudaError_t launch_eig_only(const float* S, int64_t n, float* evals, float* evec
 }
 
 cudaError_t launch_eig_only_fallback(const float* S, int64_t n, float* evals, float* evec, bool mixed,
-                                     const Fallback& fb, int64_t max_items, cudaStream_t st) {
+                                     const Fallback& fb, int64_t max_items, const Queue& st) {
   if (max_items <= 0) return cudaSuccess;
-  k_eig_only_fallback<<<fallback_grid(max_items), 128, 0, st>>>(S, n, evals, evec, mixed, fb);
-  return cudaGetLastError();
+  return launch_after(k_eig_only_fallback, fallback_grid(max_items), 128, 0, st, S, n, evals, evec, mixed, fb);
 }
 
 template <int VT, int AT, int FT, bool PLAIN, int V, typename IT>

@@ -214,7 +214,9 @@ __device__ __forceinline__ void grad_xy_body(const uint16_t* __restrict__ vol, c
 template <int RS, int XT>
 __global__ void __launch_bounds__(XT, 512 / XT)
     k_grad_xy(const uint16_t* __restrict__ vol, Box vb, int dimx, int dimy, float* __restrict__ F, Box ab, int seg,
-              const Taps tx, const Taps ty) {
+              const Taps tx, const Taps ty, int* __restrict__ zero) {
+  after_previous();
+  if (zero != nullptr && (blockIdx.x | blockIdx.y | blockIdx.z | threadIdx.x) == 0) *zero = 0;
   using G = GXYGeom<RS, XT>;
   constexpr int TB = G::TB;
   extern __shared__ __align__(16) float gsm[];
@@ -511,6 +513,7 @@ __global__ void __launch_bounds__(kGzThreads, CT_GZ_MINB > 0 ? CT_GZ_MINB : (RS 
     k_grad_z(const float* __restrict__ F, const __grid_constant__ Box ab, void* __restrict__ Jv,
              const __grid_constant__ Box ob, int seg,
              const __grid_constant__ Taps taps, const __grid_constant__ ProdScale ps) {
+  after_previous();
   grad_z_body<RS, MIXED, GOUT>(F, ab, Jv, ob, seg, taps, ps, HwBlock{});
 }
 
@@ -566,14 +569,16 @@ int sigma_kernel_radius(int r) {
   return -1;
 }
 
-cudaError_t prepare_grad_split_kernels() {
-  cudaError_t e = prepare_gs<2>();
-  if (e == cudaSuccess) e = prepare_gs<3>();
-  if (e == cudaSuccess) e = prepare_gs<4>();
-  if (e == cudaSuccess) e = prepare_gs<6>();
-  if (e == cudaSuccess) e = prepare_gs<8>();
-  if (e == cudaSuccess) e = prepare_gs<12>();
-  return e;
+cudaError_t prepare_grad_split_kernels(int rk) {
+  switch (rk) {
+    case 2: return prepare_gs<2>();
+    case 3: return prepare_gs<3>();
+    case 4: return prepare_gs<4>();
+    case 6: return prepare_gs<6>();
+    case 8: return prepare_gs<8>();
+    case 12: return prepare_gs<12>();
+    default: return cudaErrorInvalidValue;
+  }
 }
 
 // The box of the partial fields for gradient outputs over ob: ob grown by RS
@@ -589,7 +594,7 @@ Box grad_partial_box(const Box& ob, const Box& vb, int rs, int dimz) {
 
 template <int RS, int XT>
 static cudaError_t launch_gxy_t(const uint16_t* vol, const Box& vb, const int dims[3], float* F, const Box& ab,
-                                const Taps& tx, const Taps& ty, cudaStream_t st) {
+                                const Taps& tx, const Taps& ty, int* zero, const Queue& st) {
   using G = GXYGeom<RS, XT>;
   if (ab.n[2] > 65535) return cudaErrorInvalidValue;
   static int sms = 1;
@@ -599,8 +604,7 @@ static cudaError_t launch_gxy_t(const uint16_t* vol, const Box& vb, const int di
   const int seg = walk_segment(ctas, ab.n[1], G::TB, 0.5 * G::W * G::TB, slots, sms);
   dim3 grid((ab.n[0] + XT - 1) / XT, ab.n[2], (ab.n[1] + seg - 1) / seg);
   if (grid.z > 65535) return cudaErrorInvalidValue;
-  k_grad_xy<RS, XT><<<grid, XT, G::SMEM, st>>>(vol, vb, dims[0], dims[1], F, ab, seg, tx, ty);
-  return cudaGetLastError();
+  return launch_after(k_grad_xy<RS, XT>, grid, XT, G::SMEM, st, vol, vb, dims[0], dims[1], F, ab, seg, tx, ty, zero);
 }
 
 // The CTA width (columns) that covers a row of n0 with the least work: the
@@ -623,19 +627,19 @@ int cta_width(int n0, int halo, double stage, const int* widths, int n) {
 // now two of 96.
 template <int RS>
 static cudaError_t launch_gxy_r(const uint16_t* vol, const Box& vb, const int dims[3], float* F, const Box& ab,
-                                const Taps& tx, const Taps& ty, cudaStream_t st) {
+                                const Taps& tx, const Taps& ty, int* zero, const Queue& st) {
   static const int widths[] = {CT_GXY_XT, 96, 64, 160};
   switch (cta_width(ab.n[0], GXYGeom<RS, CT_GXY_XT>::XA, 0.3, widths, 4)) {
-    case 64: return launch_gxy_t<RS, 64>(vol, vb, dims, F, ab, tx, ty, st);
-    case 96: return launch_gxy_t<RS, 96>(vol, vb, dims, F, ab, tx, ty, st);
-    case 160: return launch_gxy_t<RS, 160>(vol, vb, dims, F, ab, tx, ty, st);
-    default: return launch_gxy_t<RS, CT_GXY_XT>(vol, vb, dims, F, ab, tx, ty, st);
+    case 64: return launch_gxy_t<RS, 64>(vol, vb, dims, F, ab, tx, ty, zero, st);
+    case 96: return launch_gxy_t<RS, 96>(vol, vb, dims, F, ab, tx, ty, zero, st);
+    case 160: return launch_gxy_t<RS, 160>(vol, vb, dims, F, ab, tx, ty, zero, st);
+    default: return launch_gxy_t<RS, CT_GXY_XT>(vol, vb, dims, F, ab, tx, ty, zero, st);
   }
 }
 
 template <int RS, bool MIXED, bool GOUT>
 static cudaError_t launch_gz_t(const float* F, const Box& ab, void* J, const Box& ob, const Taps& taps,
-                               const ProdScale& ps, cudaStream_t st) {
+                               const ProdScale& ps, const Queue& st) {
   static int sms = 1;
   static const int slots = resident_ctas(k_grad_z<RS, MIXED, GOUT>, kGzThreads, gz_smem<RS>(), &sms);
   const int blocks = (ob.n[0] * ob.n[1] + kGzThreads - 1) / kGzThreads;
@@ -643,13 +647,12 @@ static cudaError_t launch_gz_t(const float* F, const Box& ab, void* J, const Box
   const int seg = walk_segment(blocks, ob.n[2], 1, 0.4 * (2 * RS), slots, sms);
   const dim3 grid(blocks, 1, (ob.n[2] + seg - 1) / seg);
   if (grid.z > 65535) return cudaErrorInvalidValue;
-  k_grad_z<RS, MIXED, GOUT><<<grid, kGzThreads, gz_smem<RS>(), st>>>(F, ab, J, ob, seg, taps, ps);
-  return cudaGetLastError();
+  return launch_after(k_grad_z<RS, MIXED, GOUT>, grid, kGzThreads, gz_smem<RS>(), st, F, ab, J, ob, seg, taps, ps);
 }
 
 template <int RS>
 static cudaError_t launch_gz_r(const float* F, const Box& ab, void* J, const Box& ob, const Taps& taps,
-                               const ProdScale& ps, bool mixed, bool gout, cudaStream_t st) {
+                               const ProdScale& ps, bool mixed, bool gout, const Queue& st) {
   if (gout)
     return mixed ? launch_gz_t<RS, true, true>(F, ab, J, ob, taps, ps, st)
                  : launch_gz_t<RS, false, true>(F, ab, J, ob, taps, ps, st);
@@ -658,16 +661,16 @@ static cudaError_t launch_gz_r(const float* F, const Box& ab, void* J, const Box
 }
 
 cudaError_t launch_grad_xy(const uint16_t* vol, const Box& vb, const int dims[3], float* F, const Box& ab,
-                           const Taps& tx, const Taps& ty, int rk, cudaStream_t st) {
+                           const Taps& tx, const Taps& ty, int rk, int* zero, const Queue& st) {
   if (box_vox(ab) == 0) return cudaSuccess;
   if (box_vox(ab) >= ((int64_t)1 << 31)) return cudaErrorInvalidValue;
   switch (rk) {
-    case 2: return launch_gxy_r<2>(vol, vb, dims, F, ab, tx, ty, st);
-    case 3: return launch_gxy_r<3>(vol, vb, dims, F, ab, tx, ty, st);
-    case 4: return launch_gxy_r<4>(vol, vb, dims, F, ab, tx, ty, st);
-    case 6: return launch_gxy_r<6>(vol, vb, dims, F, ab, tx, ty, st);
-    case 8: return launch_gxy_r<8>(vol, vb, dims, F, ab, tx, ty, st);
-    case 12: return launch_gxy_r<12>(vol, vb, dims, F, ab, tx, ty, st);
+    case 2: return launch_gxy_r<2>(vol, vb, dims, F, ab, tx, ty, zero, st);
+    case 3: return launch_gxy_r<3>(vol, vb, dims, F, ab, tx, ty, zero, st);
+    case 4: return launch_gxy_r<4>(vol, vb, dims, F, ab, tx, ty, zero, st);
+    case 6: return launch_gxy_r<6>(vol, vb, dims, F, ab, tx, ty, zero, st);
+    case 8: return launch_gxy_r<8>(vol, vb, dims, F, ab, tx, ty, zero, st);
+    case 12: return launch_gxy_r<12>(vol, vb, dims, F, ab, tx, ty, zero, st);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -768,7 +771,7 @@ cudaError_t launch_grad_z_multi(const GzItem* items, const MultiTable& T, int64_
 }
 
 cudaError_t launch_grad_z(const float* F, const Box& ab, void* J, const Box& ob, const Taps& tz,
-                          const float scale[6], int rk, bool mixed, bool gout, cudaStream_t st) {
+                          const float scale[6], int rk, bool mixed, bool gout, const Queue& st) {
   if (box_vox(ob) == 0) return cudaSuccess;
   if (box_vox(ab) >= ((int64_t)1 << 31) || box_vox(ob) >= ((int64_t)1 << 31)) return cudaErrorInvalidValue;
   ProdScale ps;

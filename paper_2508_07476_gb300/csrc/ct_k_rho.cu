@@ -44,6 +44,7 @@ constexpr int kRxThreads = 6 * kRxRows * (kRxOut / kRxPer);
 template <int RR>
 __global__ void __launch_bounds__(kRxThreads, CT_RX_MINB)
     k_rho_x(const float* __restrict__ in, Box ib, int dimx, float* __restrict__ out, Box ob, const Taps taps) {
+  after_previous();
   constexpr int W = kRxOut + 2 * RR;  // staged row length (multiple of 4 for even RR)
   static_assert(W % 4 == 0, "row stride must allow 16-byte loads");
   __shared__ __align__(16) float sin_[6][kRxRows][W];
@@ -262,6 +263,7 @@ template <int RR, int kT>
 __global__ void __launch_bounds__(kStreamThreads, CT_RZ_MINB)
     k_rho_stream(const float* __restrict__ in, Box ib, int dim_axis, float* __restrict__ out, Box ob, int axis,
                  int seg, const Taps taps) {
+  after_previous();
   rho_stream_body<RR, kT>(in, ib, dim_axis, out, ob, axis, seg, taps, HwBlock{});
 }
 
@@ -277,14 +279,13 @@ __global__ void __launch_bounds__(kStreamThreads, CT_RZ_MINB)
 
 template <int RR>
 static cudaError_t launch_rho_x_r(const float* in, const Box& ib, const int dims[3], float* out, const Box& ob,
-                                  const Taps& taps, cudaStream_t st) {
+                                  const Taps& taps, const Queue& st) {
   dim3 grid((ob.n[1] * ob.n[2] + kRxRows - 1) / kRxRows, (ob.n[0] + kRxOut - 1) / kRxOut);
-  k_rho_x<RR><<<grid, kRxThreads, 0, st>>>(in, ib, dims[0], out, ob, taps);
-  return cudaGetLastError();
+  return launch_after(k_rho_x<RR>, grid, kRxThreads, 0, st, in, ib, dims[0], out, ob, taps);
 }
 
 cudaError_t launch_rho_x(const float* in, const Box& ib, const int dims[3], float* out, const Box& ob,
-                         const Taps& taps, int rk, cudaStream_t st) {
+                         const Taps& taps, int rk, const Queue& st) {
   if (box_vox(ob) == 0) return cudaSuccess;
   if ((ob.n[0] + kRxOut - 1) / kRxOut > 65535) return cudaErrorInvalidValue;
   switch (rk) {
@@ -345,6 +346,7 @@ __global__ void __launch_bounds__(kZ2Threads, RR >= 32 ? 2 : 3)
     k_rho_z2(const float* __restrict__ in, int64_t in_vox, int a_in, int n_in, int dimz, int in_row, int in_plane,
              float* __restrict__ out, int64_t out_vox, int a_out, int n_out, int out_row, int out_plane, int seg,
              const __grid_constant__ Taps taps) {
+  after_previous();
   constexpr int kT = kZ2Outputs;
   constexpr int WN = kT + 2 * RR;
   __shared__ __align__(16) float2 ring[2 * kT][kZ2Threads];
@@ -424,7 +426,7 @@ __global__ void __launch_bounds__(kZ2Threads, RR >= 32 ? 2 : 3)
 
 template <int RR, bool DENSE8>
 static cudaError_t launch_z2_t(const float* in, const Box& ib, int dimz, float* out, const Box& ob, const Taps& taps,
-                               cudaStream_t st) {
+                               const Queue& st) {
   static int sms = 1;
   static const int slots = resident_ctas(k_rho_z2<RR, DENSE8>, kZ2Threads, 0, &sms);
   const int plane = ib.n[0] * ib.n[1];
@@ -433,10 +435,8 @@ static cudaError_t launch_z2_t(const float* in, const Box& ib, int dimz, float* 
   const int seg = walk_segment((int64_t)blocks * 6, ob.n[2], kZ2Outputs, 0.25 * (2 * RR), slots, sms);
   dim3 grid(blocks, 6, (ob.n[2] + seg - 1) / seg);
   if (grid.z > 65535) return cudaErrorInvalidValue;
-  k_rho_z2<RR, DENSE8><<<grid, kZ2Threads, 0, st>>>(in, box_vox(ib), ib.lo[2], ib.n[2], dimz, ib.n[0], plane, out,
-                                                    box_vox(ob), ob.lo[2], ob.n[2], ob.n[0], ob.n[0] * ob.n[1], seg,
-                                                    taps);
-  return cudaGetLastError();
+  return launch_after(k_rho_z2<RR, DENSE8>, grid, kZ2Threads, 0, st, in, box_vox(ib), ib.lo[2], ib.n[2], dimz, ib.n[0],
+                      plane, out, box_vox(ob), ob.lo[2], ob.n[2], ob.n[0], ob.n[0] * ob.n[1], seg, taps);
 }
 
 // Whether k_rho_z2 takes the z pass: the output's columns are the first ones of
@@ -448,14 +448,14 @@ static bool z2_ok(const float* in, const Box& ib, const Box& ob) {
 
 template <int RR>
 static cudaError_t launch_z2_r(const float* in, const Box& ib, int dimz, float* out, const Box& ob, const Taps& taps,
-                               cudaStream_t st) {
+                               const Queue& st) {
   return ob.n[0] % 2 == 0 && (uintptr_t)out % 8 == 0 ? launch_z2_t<RR, true>(in, ib, dimz, out, ob, taps, st)
                                                      : launch_z2_t<RR, false>(in, ib, dimz, out, ob, taps, st);
 }
 
 template <int RR>
 static cudaError_t launch_stream_r(const float* in, const Box& ib, const int dims[3], float* out, const Box& ob,
-                                   int axis, const Taps& taps, int block_t, cudaStream_t st) {
+                                   int axis, const Taps& taps, int block_t, const Queue& st) {
   const int other = 3 - axis;
   const int n_axis = ob.n[axis];
   if (box_vox(ib) >= ((int64_t)1 << 31) || box_vox(ob) >= ((int64_t)1 << 31)) return cudaErrorInvalidValue;
@@ -464,11 +464,8 @@ static cudaError_t launch_stream_r(const float* in, const Box& ib, const int dim
   const dim3 block = rho_stream_block(ob, axis);
   dim3 grid((ob.n[0] + block.x - 1) / block.x, (6 * ob.n[other] + block.y - 1) / block.y, (n_axis + seg - 1) / seg);
   if (grid.y > 65535 || grid.z > 65535) return cudaErrorInvalidValue;
-  if (block_t == 8)
-    k_rho_stream<RR, 8><<<grid, block, 0, st>>>(in, ib, dims[axis], out, ob, axis, seg, taps);
-  else
-    k_rho_stream<RR, 16><<<grid, block, 0, st>>>(in, ib, dims[axis], out, ob, axis, seg, taps);
-  return cudaGetLastError();
+  return launch_after(block_t == 8 ? k_rho_stream<RR, 8> : k_rho_stream<RR, 16>, grid, block, 0, st, in, ib, dims[axis],
+                      out, ob, axis, seg, taps);
 }
 
 // ---------------------------------------------------------------- batches
@@ -508,7 +505,7 @@ cudaError_t launch_rho_z_multi(const RzItem* items, const MultiTable& T, int64_t
 }
 
 cudaError_t launch_rho_stream(const float* in, const Box& ib, const int dims[3], float* out, const Box& ob, int axis,
-                              const Taps& taps, int rk, int block_t, cudaStream_t st) {
+                              const Taps& taps, int rk, int block_t, const Queue& st) {
   if (box_vox(ob) == 0) return cudaSuccess;
   if (axis != 1 && axis != 2) return cudaErrorInvalidValue;
   switch (rk) {

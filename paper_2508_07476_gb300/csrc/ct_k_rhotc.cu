@@ -447,6 +447,7 @@ __global__ void __launch_bounds__(TcRoles<XAXIS, PROD>::THREADS, 1)
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  after_previous();  // the taps' matrix, the barriers and the tensor memory are set up before
   const uint32_t tm = tmem_base;
   const uint32_t tlane = tm + ((uint32_t)(wq * 32) << 16);  // this warp's 32 lanes
   // mbarriers of tile g, and the parity of its phase
@@ -989,7 +990,7 @@ struct TcLaunch {
     return cudaSuccess;
   }
   static cudaError_t run(const float* in, const Box& ib, const int dims[3], float* out, const Box& ob, int axis,
-                         const Taps& taps, const TcCtl& ctl, const TcProd& pr, cudaStream_t st) {
+                         const Taps& taps, const TcCtl& ctl, const TcProd& pr, const Queue& st) {
     using G = TcGeom<RR>;
     cudaError_t e = prepare();
     if (e != cudaSuccess) return e;
@@ -1030,10 +1031,8 @@ struct TcLaunch {
       if (vin && ob.lo[1] == ib.lo[1] && ob.n[1] == ib.n[1] && rows_map(&tin, in, ib)) flags |= 4;
       if (vout && rows_map(&tout, out, ob)) flags |= 8;
     }
-    k_rho_tc<RR, XAXIS, PROD><<<grid, TcRoles<XAXIS, PROD>::THREADS, G::smem(XAXIS, PROD), st>>>(in, ib, dims[axis], out, ob,
-                                                                                           axis, seg,
-                                                                              flags, taps, tin, tout, ctl, pr);
-    return cudaGetLastError();
+    return launch_after(k_rho_tc<RR, XAXIS, PROD>, grid, TcRoles<XAXIS, PROD>::THREADS, G::smem(XAXIS, PROD), st, in, ib,
+                        dims[axis], out, ob, axis, seg, flags, taps, tin, tout, ctl, pr);
   }
 };
 template <int RR, bool XAXIS, int PROD>
@@ -1041,7 +1040,7 @@ bool TcLaunch<RR, XAXIS, PROD>::ready = false;
 
 template <int RR>
 cudaError_t run_tc(const float* in, const Box& ib, const int dims[3], float* out, const Box& ob, int axis,
-                   const Taps& taps, const TcCtl& ctl, int prod, const TcProd& pr, cudaStream_t st) {
+                   const Taps& taps, const TcCtl& ctl, int prod, const TcProd& pr, const Queue& st) {
   if (axis == 0) return TcLaunch<RR, true, 0>::run(in, ib, dims, out, ob, axis, taps, ctl, pr, st);
   if (prod == 1) return TcLaunch<RR, false, 1>::run(in, ib, dims, out, ob, axis, taps, ctl, pr, st);
   if (prod == 2) return TcLaunch<RR, false, 2>::run(in, ib, dims, out, ob, axis, taps, ctl, pr, st);
@@ -1058,7 +1057,7 @@ cudaError_t prepare_tc() {
 }
 
 cudaError_t dispatch_tc(const float* in, const Box& ib, const int dims[3], float* out, const Box& ob, int axis,
-                        const Taps& taps, int rk, const TcCtl& ctl, int prod, const TcProd& pr, cudaStream_t st) {
+                        const Taps& taps, int rk, const TcCtl& ctl, int prod, const TcProd& pr, const Queue& st) {
   if (box_vox(ob) == 0) return cudaSuccess;
   if (axis < 0 || axis > 2 || (prod && axis == 0)) return cudaErrorInvalidValue;
   switch (rk) {
@@ -1076,20 +1075,22 @@ cudaError_t dispatch_tc(const float* in, const Box& ib, const int dims[3], float
 
 }  // namespace
 
-cudaError_t prepare_rho_tc_kernels() {
-  cudaError_t e = prepare_tc<4>();
-  if (e == cudaSuccess) e = prepare_tc<6>();
-  if (e == cudaSuccess) e = prepare_tc<8>();
-  if (e == cudaSuccess) e = prepare_tc<12>();
-  if (e == cudaSuccess) e = prepare_tc<16>();
-  if (e == cudaSuccess) e = prepare_tc<24>();
-  if (e == cudaSuccess) e = prepare_tc<32>();
-  if (e == cudaSuccess) e = prepare_tc<36>();
-  return e;
+cudaError_t prepare_rho_tc_kernels(int rk) {
+  switch (rk) {
+    case 4: return prepare_tc<4>();
+    case 6: return prepare_tc<6>();
+    case 8: return prepare_tc<8>();
+    case 12: return prepare_tc<12>();
+    case 16: return prepare_tc<16>();
+    case 24: return prepare_tc<24>();
+    case 32: return prepare_tc<32>();
+    case 36: return prepare_tc<36>();
+    default: return cudaErrorInvalidValue;
+  }
 }
 
 cudaError_t launch_rho_tc(const float* in, const Box& ib, const int dims[3], float* out, const Box& ob, int axis,
-                          const Taps& taps, int rk, const TcCtl& ctl, cudaStream_t st) {
+                          const Taps& taps, int rk, const TcCtl& ctl, const Queue& st) {
   TcProd pr;
   std::memset(&pr, 0, sizeof pr);
   return dispatch_tc(in, ib, dims, out, ob, axis, taps, rk, ctl, 0, pr, st);
@@ -1097,7 +1098,7 @@ cudaError_t launch_rho_tc(const float* in, const Box& ib, const int dims[3], flo
 
 cudaError_t launch_rho_tc_products(const void* g, bool half, const Box& ib, const int dims[3], float* out,
                                    const Box& ob, int axis, const Taps& taps, const float scale[6], int rk,
-                                   const TcCtl& ctl, cudaStream_t st) {
+                                   const TcCtl& ctl, const Queue& st) {
   TcProd pr;
   pr.unit = 1;
   for (int k = 0; k < 6; ++k) {

@@ -214,6 +214,7 @@ template <int RR, int XT, bool SAMEXY>
 __global__ void __launch_bounds__(XT, CT_XY_MINB * 256 / XT)
     k_rho_xy(const float* __restrict__ in, Box ib, int dimx, int dimy, float* __restrict__ out, Box ob, int seg,
              const Taps tx, const Taps ty) {
+  after_previous();
   using G = XYGeom<RR, XT>;
   constexpr int kTB = G::TB;
   constexpr int kXT = XT;
@@ -381,7 +382,7 @@ __global__ void __launch_bounds__(XT, CT_XY_MINB * 256 / XT)
 
 template <int RR, int XT, bool SAME>
 static cudaError_t launch_xy_rt(const float* in, const Box& ib, const int dims[3], float* out, const Box& ob,
-                                const Taps& tx, const Taps& ty, cudaStream_t st) {
+                                const Taps& tx, const Taps& ty, const Queue& st) {
   using G = XYGeom<RR, XT>;
   constexpr int kTB = G::TB;
   const size_t smem = sizeof(float) * (kStages * kTB * G::XS + kTB * G::SXS);
@@ -394,8 +395,7 @@ static cudaError_t launch_xy_rt(const float* in, const Box& ib, const int dims[3
   const int seg = walk_segment(ctas, ob.n[1], kTB, 0.6 * G::W * kTB, slots, sms);
   dim3 grid((ob.n[0] + XT - 1) / XT, (unsigned)rows, (ob.n[1] + seg - 1) / seg);
   if (grid.z > 65535) return cudaErrorInvalidValue;
-  k_rho_xy<RR, XT, SAME><<<grid, XT, smem, st>>>(in, ib, dims[0], dims[1], out, ob, seg, tx, ty);
-  return cudaGetLastError();
+  return launch_after(k_rho_xy<RR, XT, SAME>, grid, XT, smem, st, in, ib, dims[0], dims[1], out, ob, seg, tx, ty);
 }
 
 // 128-column CTAs when they leave fewer idle columns than 256-column ones.
@@ -406,7 +406,7 @@ static bool narrow_xy(int n0) {
 
 template <int RR>
 static cudaError_t launch_xy_r(const float* in, const Box& ib, const int dims[3], float* out, const Box& ob,
-                               const Taps& tx, const Taps& ty, cudaStream_t st) {
+                               const Taps& tx, const Taps& ty, const Queue& st) {
   if (box_vox(ib) >= ((int64_t)1 << 31) || box_vox(ob) >= ((int64_t)1 << 31)) return cudaErrorInvalidValue;
   if (std::memcmp(&tx, &ty, sizeof(Taps)) != 0)  // anisotropic voxels: two tap sets
     return narrow_xy(ob.n[0]) ? launch_xy_rt<RR, 128, false>(in, ib, dims, out, ob, tx, ty, st)
@@ -457,16 +457,18 @@ static cudaError_t prepare_xy_r() {
   return e;
 }
 
-cudaError_t prepare_rho_xy_kernels() {
-  cudaError_t e = prepare_xy_r<4>();
-  if (e == cudaSuccess) e = prepare_xy_r<6>();
-  if (e == cudaSuccess) e = prepare_xy_r<8>();
-  if (e == cudaSuccess) e = prepare_xy_r<12>();
-  if (e == cudaSuccess) e = prepare_xy_r<16>();
-  if (e == cudaSuccess) e = prepare_xy_r<24>();
-  if (e == cudaSuccess) e = prepare_xy_r<32>();
-  if (e == cudaSuccess) e = prepare_xy_r<36>();
-  return e;
+cudaError_t prepare_rho_xy_kernels(int rk) {
+  switch (rk) {
+    case 4: return prepare_xy_r<4>();
+    case 6: return prepare_xy_r<6>();
+    case 8: return prepare_xy_r<8>();
+    case 12: return prepare_xy_r<12>();
+    case 16: return prepare_xy_r<16>();
+    case 24: return prepare_xy_r<24>();
+    case 32: return prepare_xy_r<32>();
+    case 36: return prepare_xy_r<36>();
+    default: return cudaErrorInvalidValue;
+  }
 }
 
 // ---------------------------------------------------------------- batches
@@ -536,7 +538,7 @@ cudaError_t launch_rho_xy_multi(const RxyItem* items, const MultiTable& T, int64
 }
 
 cudaError_t launch_rho_xy(const float* in, const Box& ib, const int dims[3], float* out, const Box& ob,
-                          const Taps& tx, const Taps& ty, int rk, cudaStream_t st) {
+                          const Taps& tx, const Taps& ty, int rk, const Queue& st) {
   if (box_vox(ob) == 0) return cudaSuccess;
   switch (rk) {
     case 4: return launch_xy_r<4>(in, ib, dims, out, ob, tx, ty, st);

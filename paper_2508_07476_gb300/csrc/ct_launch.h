@@ -11,10 +11,42 @@
 
 namespace ct {
 
-// Set the shared-memory attributes of every kernel instantiation (once per process,
-// before any launch may be captured into a graph).
-cudaError_t prepare_rho_xy_kernels();
-cudaError_t prepare_grad_split_kernels();
+// Set the shared-memory attributes of the kernel instantiations of one radius
+// (once per plan and radius, before any launch may be captured into a graph).
+cudaError_t prepare_rho_xy_kernels(int rk);
+cudaError_t prepare_grad_split_kernels(int rk);
+
+// Where a kernel of the chain goes: the stream, and whether its CTAs may be
+// scheduled while the stream's previous kernel drains (`early`; every kernel
+// launched through launch_after begins with after_previous(), which waits for that
+// kernel).  That hides the launch latency of a chain of short kernels (64^3: 50 ->
+// 40 us; 173 x 141 x 118: 207 -> 195; a 256^3 chunk: 1118 -> 1099), but an SM that
+// never drains keeps its split of L1 and shared memory: the eigen stage after a
+// tensor-core pass then runs with little L1 (512^3: 4837 -> 4949 us; a 384^3 chunk,
+// 57M voxels: even), and beside other streams the waiting CTAs hold room those could
+// use (12 crops on four streams: 6.28 -> 6.41 ms).  So: boxes of at most
+// kEarlyMaxVox voxels, outside captured batches.
+constexpr int64_t kEarlyMaxVox = (int64_t)1 << 25;
+struct Queue {
+  cudaStream_t st;
+  bool early;
+  Queue(cudaStream_t s, bool e = false) : st(s), early(e) {}
+};
+
+template <typename... P, typename... A>
+cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, const Queue& q, A&&... args) {
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = q.early ? 1 : 0;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = q.st;
+  cfg.attrs = &attr;
+  cfg.numAttrs = q.early ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
 
 // How many segments to cut the walk of a streaming kernel into: `ctas` CTAs
 // walk n positions each, a segment of L of them costing L + warm (warm: the
@@ -76,22 +108,23 @@ int rho_kernel_radius(int r);
 Box grad_partial_box(const Box& ob, const Box& vb, int rs, int dimz);
 // tx / ty / tz: the taps of each axis (anisotropic voxels); scale: the factor of
 // each product (1 / (spacing_a spacing_b), xx yy zz xy xz yz).
+// zero (nullable): a device counter that the kernel clears (the eigen stage's list).
 cudaError_t launch_grad_xy(const uint16_t* vol, const Box& vb, const int dims[3], float* F, const Box& ab,
-                           const Taps& tx, const Taps& ty, int rk, cudaStream_t st);
+                           const Taps& tx, const Taps& ty, int rk, int* zero, const Queue& st);
 cudaError_t launch_grad_z(const float* F, const Box& ab, void* J, const Box& ob, const Taps& tz,
-                          const float scale[6], int rk, bool mixed, bool gout, cudaStream_t st);
+                          const float scale[6], int rk, bool mixed, bool gout, const Queue& st);
 
 // rho pass along x: out (6 planes over ob) from in (6 planes over ib).
 cudaError_t launch_rho_x(const float* in, const Box& ib, const int dims[3], float* out, const Box& ob,
-                         const Taps& taps, int rk, cudaStream_t st);
+                         const Taps& taps, int rk, const Queue& st);
 
 // rho passes along x and y fused: out (6 planes over ob) from in (6 planes over ib).
 cudaError_t launch_rho_xy(const float* in, const Box& ib, const int dims[3], float* out, const Box& ob,
-                          const Taps& tx, const Taps& ty, int rk, cudaStream_t st);
+                          const Taps& tx, const Taps& ty, int rk, const Queue& st);
 
 // rho pass along axis 1 (y) or 2 (z), streaming register windows of block_t (8 or 16) outputs.
 cudaError_t launch_rho_stream(const float* in, const Box& ib, const int dims[3], float* out, const Box& ob, int axis,
-                              const Taps& taps, int rk, int block_t, cudaStream_t st);
+                              const Taps& taps, int rk, int block_t, const Queue& st);
 
 // rho pass along axis 0, 1 or 2 on the tensor cores (banded Toeplitz product,
 // TF32 split operands, FP32 accumulation): same contract as launch_rho_x /
@@ -105,16 +138,16 @@ struct TcCtl {
   uint32_t wait_limit;
   int seg_cap;  // outputs per work unit at most (0: 512); the work is then spread over the SMs
 };
-cudaError_t prepare_rho_tc_kernels();
+cudaError_t prepare_rho_tc_kernels(int rk);
 cudaError_t launch_rho_tc(const float* in, const Box& ib, const int dims[3], float* out, const Box& ob, int axis,
-                          const Taps& taps, int rk, const TcCtl& ctl, cudaStream_t st);
+                          const Taps& taps, int rk, const TcCtl& ctl, const Queue& st);
 // The same pass along axis 1 or 2 reading the gradient instead of the tensor:
 // g (3 planes over ib: FP16 holding g * 2^-8 when half, else FP32, as
 // launch_grad_z writes them with gout) -> out (6 planes over ob) = the pass of
 // the products g_a g_b * scale[k], each formed as launch_grad_z forms it.
 cudaError_t launch_rho_tc_products(const void* g, bool half, const Box& ib, const int dims[3], float* out,
                                    const Box& ob, int axis, const Taps& taps, const float scale[6], int rk,
-                                   const TcCtl& ctl, cudaStream_t st);
+                                   const TcCtl& ctl, const Queue& st);
 // Whether a volume nx voxels wide suits launch_rho_tc along axis: 16-byte copies
 // of its rows (x extent a multiple of 4).
 bool rho_tc_volume_aligned(int nx, int axis);
@@ -233,17 +266,17 @@ cudaError_t launch_eig_fallback_multi(const EigItem* items, int n_items, int64_t
 // solves them with full warps (the same arithmetic per voxel).
 cudaError_t launch_eig_angles(const float* S, const Box& sb, const Box& ob, const uint8_t* mask, const Box& mb,
                               const Frame& F, float fill, const EigOut& o, bool mixed, const Fallback& fb,
-                              bool compact, cudaStream_t st);
+                              bool compact, const Queue& st);
 // Re-solve the listed voxels (FP32 Jacobi, or FP64 in the mixed form) and rewrite their outputs.
 cudaError_t launch_eig_angles_fallback(const float* S, const Box& sb, const Box& ob, const uint8_t* mask,
                                        const Box& mb, const Frame& F, float fill, const EigOut& o, bool mixed,
-                                       const Fallback& fb, int64_t max_items, cudaStream_t st);
+                                       const Fallback& fb, int64_t max_items, const Queue& st);
 
 // Stage kernels: eigen only (evals + unoriented evec), and angles only.
 cudaError_t launch_eig_only(const float* S, int64_t n, float* evals, float* evec, bool mixed, const Fallback& fb,
                             cudaStream_t st);
 cudaError_t launch_eig_only_fallback(const float* S, int64_t n, float* evals, float* evec, bool mixed,
-                                     const Fallback& fb, int64_t max_items, cudaStream_t st);
+                                     const Fallback& fb, int64_t max_items, const Queue& st);
 cudaError_t launch_angles_only(const float* evec, const float* evals, const Box& ob, const uint8_t* mask,
                                const Frame& F, float fill, const EigOut& o, cudaStream_t st);
 
