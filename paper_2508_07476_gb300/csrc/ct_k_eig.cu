@@ -362,6 +362,8 @@ cudaError_t launch_eig_angles(const float* S, const Box& sb, const Box& ob, cons
           return launch_after(k_eig_angles_compact<1, 1, 1, true>, gc, kEigThreads, 0, st, S, sb, ob, mask, mb, F, fill, o, mixed, fb);
         else
           return launch_after(k_eig_angles_compact<1, 1, 1, false>, gc, kEigThreads, 0, st, S, sb, ob, mask, mb, F, fill, o, mixed, fb);
+      } else if (o.vec_t == CT_OUT_F32 && o.ang_t == CT_OUT_U8Q && o.fa_t == CT_OUT_F16 && plain) {
+        return launch_after(k_eig_angles_compact<0, 2, 1, true>, gc, kEigThreads, 0, st, S, sb, ob, mask, mb, F, fill, o, mixed, fb);
       } else if (o.ang_t == CT_OUT_U8Q && o.fa_t == CT_OUT_F16) {
         return launch_after(k_eig_angles_compact<-1, 2, 1, false>, gc, kEigThreads, 0, st, S, sb, ob, mask, mb, F, fill, o, mixed, fb);
       } else {
@@ -378,6 +380,8 @@ cudaError_t launch_eig_angles(const float* S, const Box& sb, const Box& ob, cons
         return launch_after(k_eig_angles32<1, 1, 1, true>, g3, nt, 0, st, S, sb, ob, mask, mb, F, fill, o, mixed, fb);
       else
         return launch_after(k_eig_angles32<1, 1, 1, false>, g3, nt, 0, st, S, sb, ob, mask, mb, F, fill, o, mixed, fb);
+    } else if (o.vec_t == CT_OUT_F32 && o.ang_t == CT_OUT_U8Q && o.fa_t == CT_OUT_F16 && plain) {
+      return launch_after(k_eig_angles32<0, 2, 1, true>, g3, nt, 0, st, S, sb, ob, mask, mb, F, fill, o, mixed, fb);
     } else if (o.ang_t == CT_OUT_U8Q && o.fa_t == CT_OUT_F16) {
       return launch_after(k_eig_angles32<-1, 2, 1, false>, g3, nt, 0, st, S, sb, ob, mask, mb, F, fill, o, mixed, fb);
     } else {

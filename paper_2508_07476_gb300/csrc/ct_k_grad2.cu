@@ -58,7 +58,16 @@ struct GXYGeom {
   static constexpr int B2 = OFF / 2 * 2, O2 = OFF % 2;     // 16-byte aligned start (2 voxels), remainder
   static constexpr int NV = (XH + 2 * RS + O2 + 1) / 2;    // float4 loads (2 voxel pairs each) per sub-pass
   static constexpr size_t SMEM = sizeof(float) * (TB * XS + TB * SXS);
+  // The single-item kernel with slots (SLOTS): its 16-byte chunks come by cp.async
+  // into slots of their own threads, two blocks ahead, instead of into registers one
+  // block ahead, where they were waited for.
+  static constexpr int RAW = 3;  // blocks of slots
+  static constexpr size_t SMEM_SLOTS = SMEM + (size_t)RAW * NQ * XT * sizeof(uint4);
 };
+
+__device__ __forceinline__ void cp_async16_u16(uint32_t smem_dst, const uint16_t* gsrc) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem_dst), "l"(gsrc) : "memory");
+}
 
 // 8 uint16 (one 16-byte chunk) -> 8 floats, exact.
 __device__ __forceinline__ void u16x8_to_f32(const uint4 q, float* f) {
@@ -211,7 +220,7 @@ __device__ __forceinline__ void grad_xy_body(const uint16_t* __restrict__ vol, c
 
 // The single-item kernel keeps its own copy of the body (through the body
 // function it ran 6% slower).
-template <int RS, int XT>
+template <int RS, int XT, bool SLOTS>
 __global__ void __launch_bounds__(XT, 512 / XT)
     k_grad_xy(const uint16_t* __restrict__ vol, Box vb, int dimx, int dimy, float* __restrict__ F, Box ab, int seg,
               const Taps tx, const Taps ty, int* __restrict__ zero) {
@@ -247,29 +256,38 @@ __global__ void __launch_bounds__(XT, 512 / XT)
     q_col[i] = x0 - G::XA + 8 * (q / TB);
     q_fast[i] = aligned && q_col[i] >= xlo_ok && q_col[i] + 7 < xhi_ok && ((q_col[i] - vb.lo[0]) % 8) == 0;
   }
-  uint4 pre[G::NQ];
-  auto load_block = [&](int b) {  // block b's chunks into registers
+  uint4 pre[SLOTS ? 1 : G::NQ];
+  uint4* raw = reinterpret_cast<uint4*>(gsm + TB * (G::XS + G::SXS)) + t;  // this thread's slots [RAW][NQ], XT apart
+  auto slot = [&](int b, int i) { return raw + ((b % G::RAW) * G::NQ + i) * XT; };
+  auto load_block = [&](int b) {  // block b's chunks into registers or slots
 #pragma unroll
     for (int i = 0; i < G::NQ; ++i) {
       if (q_row[i] < 0) continue;
       const int y = min(max(p0 - RS - G::PAD + b * TB + q_row[i], ylo), yhi);
       const uint16_t* row = plane + (int64_t)(y - vb.lo[1]) * vb.n[0] - vb.lo[0];
       if (q_fast[i]) {
-        pre[i] = __ldg(reinterpret_cast<const uint4*>(row + q_col[i]));
+        if (SLOTS)
+          cp_async16_u16((uint32_t)__cvta_generic_to_shared(slot(b, i)), row + q_col[i]);
+        else
+          pre[SLOTS ? 0 : i] = __ldg(reinterpret_cast<const uint4*>(row + q_col[i]));
       } else {
         uint32_t h[8];
 #pragma unroll
         for (int e = 0; e < 8; ++e) h[e] = __ldg(row + clamp_to(q_col[i] + e, dimx, vb.lo[0], vb.n[0]));
-        pre[i] = make_uint4(h[0] | (h[1] << 16), h[2] | (h[3] << 16), h[4] | (h[5] << 16), h[6] | (h[7] << 16));
+        const uint4 q = make_uint4(h[0] | (h[1] << 16), h[2] | (h[3] << 16), h[4] | (h[5] << 16), h[6] | (h[7] << 16));
+        if (SLOTS)
+          *slot(b, i) = q;
+        else
+          pre[SLOTS ? 0 : i] = q;
       }
     }
   };
-  auto store_block = [&]() {  // registers -> staged rows, every voxel twice
+  auto store_block = [&](int b) {  // registers or slots -> staged rows, every voxel twice
 #pragma unroll
     for (int i = 0; i < G::NQ; ++i) {
       if (q_row[i] < 0) continue;
       float f[8];
-      u16x8_to_f32(pre[i], f);
+      u16x8_to_f32(SLOTS ? *slot(b, i) : pre[SLOTS ? 0 : i], f);
       float4* d = reinterpret_cast<float4*>(stage + q_row[i] * G::XS + 2 * (q_col[i] - (x0 - G::XA)));
 #pragma unroll
       for (int e = 0; e < 4; ++e) d[e] = make_float4(f[2 * e], f[2 * e], f[2 * e + 1], f[2 * e + 1]);
@@ -289,10 +307,17 @@ __global__ void __launch_bounds__(XT, 512 / XT)
   const float2 cw0 = make_float2(0.f, tx.w[RS]);  // centre tap of (c_x, w_x)
   const float2 sgn = make_float2(-1.f, 1.f);
   const float2 wy0 = make_float2(ty.w[RS], ty.w[RS]);
-  load_block(0);
+  constexpr int AHEAD = SLOTS ? G::RAW - 1 : 1;  // blocks in flight during a block's passes
+#pragma unroll
+  for (int b = 0; b < AHEAD; ++b) {
+    if (b < nblocks) load_block(b);
+    if (SLOTS) cp_async_commit();
+  }
   for (int b = 0; b < nblocks; ++b) {
-    store_block();                           // the staged rows were last read before the previous barrier
-    if (b + 1 < nblocks) load_block(b + 1);  // in flight during this block's passes
+    if (SLOTS) cp_async_wait<AHEAD - 1>();  // block b has landed (this thread's own copies)
+    store_block(b);                          // the staged rows were last read before the previous barrier
+    if (b + AHEAD < nblocks) load_block(b + AHEAD);
+    if (SLOTS) cp_async_commit();
     __syncthreads();                         // staged rows complete; x-pass rows free
     // x pass: 8 outputs of row xr (+ 8 r), columns xseg*8 .. +7, in sub-passes of XH
 #pragma unroll
@@ -532,11 +557,20 @@ __global__ void __launch_bounds__(kGzThreads, CT_GZ_MINB > 0 ? CT_GZ_MINB : (RS 
 #ifndef CT_GXY_XT
 #define CT_GXY_XT 128  // columns (threads) per gradient x/y CTA (tuning choice)
 #endif
-template <int RS, int XT>
-static cudaError_t set_xy_attr() {
-  return cudaFuncSetAttribute(k_grad_xy<RS, XT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)GXYGeom<RS, XT>::SMEM);
+template <int RS, int XT, bool SLOTS>
+constexpr int gxy_smem() {
+  return (int)(SLOTS ? GXYGeom<RS, XT>::SMEM_SLOTS : GXYGeom<RS, XT>::SMEM);
 }
+
+template <int RS, int XT, bool SLOTS>
+static cudaError_t set_xy_attr() {
+  return cudaFuncSetAttribute(k_grad_xy<RS, XT, SLOTS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              gxy_smem<RS, XT, SLOTS>());
+}
+
+// R = 12 walks in short blocks of 8 rows, and the chunks' registers made it spill:
+// slots at every width (a haloed 384^3 chunk: 760 -> 694 us).
+constexpr bool gxy_slots(int rs) { return rs > 8; }
 
 template <int RS>
 static size_t gz_smem() {
@@ -545,10 +579,11 @@ static size_t gz_smem() {
 
 template <int RS>
 static cudaError_t prepare_gs() {
-  cudaError_t e = set_xy_attr<RS, CT_GXY_XT>();
-  if (e == cudaSuccess) e = set_xy_attr<RS, 64>();
-  if (e == cudaSuccess) e = set_xy_attr<RS, 96>();
-  if (e == cudaSuccess) e = set_xy_attr<RS, 160>();
+  cudaError_t e = set_xy_attr<RS, CT_GXY_XT, gxy_slots(RS)>();
+  if (e == cudaSuccess) e = set_xy_attr<RS, 64, gxy_slots(RS)>();
+  if (e == cudaSuccess) e = set_xy_attr<RS, 96, gxy_slots(RS)>();
+  if (e == cudaSuccess) e = set_xy_attr<RS, 160, gxy_slots(RS)>();
+  if (e == cudaSuccess) e = set_xy_attr<RS, CT_GXY_XT, true>();
   const int sm = (int)gz_smem<RS>();
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_grad_xy_multi<RS, CT_GXY_XT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -592,19 +627,20 @@ Box grad_partial_box(const Box& ob, const Box& vb, int rs, int dimz) {
   return a;
 }
 
-template <int RS, int XT>
+template <int RS, int XT, bool SLOTS>
 static cudaError_t launch_gxy_t(const uint16_t* vol, const Box& vb, const int dims[3], float* F, const Box& ab,
                                 const Taps& tx, const Taps& ty, int* zero, const Queue& st) {
   using G = GXYGeom<RS, XT>;
   if (ab.n[2] > 65535) return cudaErrorInvalidValue;
   static int sms = 1;
-  static const int slots = resident_ctas(k_grad_xy<RS, XT>, XT, G::SMEM, &sms);
+  static const int slots = resident_ctas(k_grad_xy<RS, XT, SLOTS>, XT, gxy_smem<RS, XT, SLOTS>(), &sms);
   const int64_t ctas = (int64_t)((ab.n[0] + XT - 1) / XT) * ab.n[2];
   // a warm-up block stages its rows and filters them along x
   const int seg = walk_segment(ctas, ab.n[1], G::TB, 0.5 * G::W * G::TB, slots, sms);
   dim3 grid((ab.n[0] + XT - 1) / XT, ab.n[2], (ab.n[1] + seg - 1) / seg);
   if (grid.z > 65535) return cudaErrorInvalidValue;
-  return launch_after(k_grad_xy<RS, XT>, grid, XT, G::SMEM, st, vol, vb, dims[0], dims[1], F, ab, seg, tx, ty, zero);
+  return launch_after(k_grad_xy<RS, XT, SLOTS>, grid, XT, gxy_smem<RS, XT, SLOTS>(), st, vol, vb, dims[0], dims[1], F, ab,
+                      seg, tx, ty, zero);
 }
 
 // The CTA width (columns) that covers a row of n0 with the least work: the
@@ -629,11 +665,18 @@ template <int RS>
 static cudaError_t launch_gxy_r(const uint16_t* vol, const Box& vb, const int dims[3], float* F, const Box& ab,
                                 const Taps& tx, const Taps& ty, int* zero, const Queue& st) {
   static const int widths[] = {CT_GXY_XT, 96, 64, 160};
-  switch (cta_width(ab.n[0], GXYGeom<RS, CT_GXY_XT>::XA, 0.3, widths, 4)) {
-    case 64: return launch_gxy_t<RS, 64>(vol, vb, dims, F, ab, tx, ty, zero, st);
-    case 96: return launch_gxy_t<RS, 96>(vol, vb, dims, F, ab, tx, ty, zero, st);
-    case 160: return launch_gxy_t<RS, 160>(vol, vb, dims, F, ab, tx, ty, zero, st);
-    default: return launch_gxy_t<RS, CT_GXY_XT>(vol, vb, dims, F, ab, tx, ty, zero, st);
+  const int w = cta_width(ab.n[0], GXYGeom<RS, CT_GXY_XT>::XA, 0.3, widths, 4);
+  // Slots for large boxes of whole 16-byte chunks too (512^3, R = 8: 616 -> 576 us).
+  // Ragged rows go through registers either way, and beside other kernels the slots'
+  // shared memory costs more than it gives (12 uneven crops 6.24 -> 6.39 ms, a 256^3
+  // chunk 1098 -> 1103 us).
+  if (w == CT_GXY_XT && box_vox(ab) > kEarlyMaxVox && vb.n[0] % 8 == 0 && (uintptr_t)vol % 16 == 0)
+    return launch_gxy_t<RS, CT_GXY_XT, true>(vol, vb, dims, F, ab, tx, ty, zero, st);
+  switch (w) {
+    case 64: return launch_gxy_t<RS, 64, gxy_slots(RS)>(vol, vb, dims, F, ab, tx, ty, zero, st);
+    case 96: return launch_gxy_t<RS, 96, gxy_slots(RS)>(vol, vb, dims, F, ab, tx, ty, zero, st);
+    case 160: return launch_gxy_t<RS, 160, gxy_slots(RS)>(vol, vb, dims, F, ab, tx, ty, zero, st);
+    default: return launch_gxy_t<RS, CT_GXY_XT, gxy_slots(RS)>(vol, vb, dims, F, ab, tx, ty, zero, st);
   }
 }
 

@@ -411,16 +411,16 @@ static cudaError_t launch_xy_r(const float* in, const Box& ib, const int dims[3]
   if (std::memcmp(&tx, &ty, sizeof(Taps)) != 0)  // anisotropic voxels: two tap sets
     return narrow_xy(ob.n[0]) ? launch_xy_rt<RR, 128, false>(in, ib, dims, out, ob, tx, ty, st)
                               : launch_xy_rt<RR, 256, false>(in, ib, dims, out, ob, tx, ty, st);
-  // the width with the fewest idle columns (they filter like the others); a staged
-  // column beside the CTA's own costs a tenth of one (0.02 .. 0.25 choose alike
-  // but for narrow rows): 173 columns in two CTAs of 96 instead of one of 256
-  static const int widths[] = {256, 128, 96, 64, 160};
-  switch (cta_width(ob.n[0], RR, 0.1, widths, 5)) {
+  // The width with the fewest idle columns (they filter like the others); a staged
+  // column beside the CTA's own costs a tenth of one.  173 columns at R = 16: two CTAs of
+  // 96 84 us, three of 64 85, one of 256 129; 250 columns at R = 24: two of 128 272 us, one of
+  // 256 280, four of 64 326; 12 uneven crops 6.24 ms at this weight, 6.40 at 0.6.
+  static const int widths[] = {128, 96, 64, 160};
+  switch (cta_width(ob.n[0], RR, 0.1, widths, 4)) {
     case 64: return launch_xy_rt<RR, 64, true>(in, ib, dims, out, ob, tx, ty, st);
     case 96: return launch_xy_rt<RR, 96, true>(in, ib, dims, out, ob, tx, ty, st);
-    case 128: return launch_xy_rt<RR, 128, true>(in, ib, dims, out, ob, tx, ty, st);
     case 160: return launch_xy_rt<RR, 160, true>(in, ib, dims, out, ob, tx, ty, st);
-    default: return launch_xy_rt<RR, 256, true>(in, ib, dims, out, ob, tx, ty, st);
+    default: return launch_xy_rt<RR, 128, true>(in, ib, dims, out, ob, tx, ty, st);
   }
 }
 
@@ -438,8 +438,9 @@ static cudaError_t prepare_xy_1() {
 template <int RR, int XT>
 static cudaError_t prepare_xy_rt() {
   constexpr int smem = xy_smem<RR, XT>();
-  cudaError_t e = prepare_xy_1<RR, XT, true>();
-  if (e == cudaSuccess) e = prepare_xy_1<RR, XT, false>();
+  cudaError_t e = prepare_xy_1<RR, XT, false>();
+  if constexpr (XT != 256)
+    if (e == cudaSuccess) e = prepare_xy_1<RR, XT, true>();
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_rho_xy_multi<RR, XT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e == cudaSuccess)
