@@ -152,6 +152,41 @@ __global__ void __launch_bounds__(256, CT_EIG_MINB)
   eig32_body<VT, AT, FT, PLAIN>(S, sb, ob, mask, mb, F, fill, o, fb, HwBlock{});
 }
 
+// The unmasked form: a CTA of kEigRowThreads threads takes up to kEigRowSpan
+// consecutive voxels of one row in a loop, so that the row's part of the indices
+// and of the frame, and the kernel's set-up, are paid once per CTA and not once
+// per voxel.  The solve is bound by its instructions (about 400 per voxel, 87% of
+// the issue slots): 173 x 141 x 118 45.0 us with a voxel per thread, 40.8 so; 12 uneven
+// crops 6.26 -> 6.17 ms (spans of 4 voxels per thread 6.21, of 2 6.29; 32 or 20 CTAs
+// per SM instead of 24, at 32 / 42 registers: 6.24).
+constexpr int kEigRowThreads = 64;
+constexpr int kEigRowSpan = 8 * kEigRowThreads;
+template <int VT, int AT, int FT, bool PLAIN>
+__global__ void __launch_bounds__(kEigRowThreads, 24)
+    k_eig_angles_rows(const float* __restrict__ S, Box sb, Box ob, Frame F, float fill, EigOut o, Fallback fb) {
+  after_previous();
+  const int y = ob.lo[1] + blockIdx.y, z = ob.lo[2] + blockIdx.z;
+  const int x0 = ob.lo[0] + blockIdx.x * kEigRowSpan;
+  const int xend = min(ob.lo[0] + ob.n[0], x0 + kEigRowSpan);
+  const int ns = sb.n[0] * sb.n[1] * sb.n[2];
+  const float* p = S + box_index32(sb, x0, y, z) + threadIdx.x;
+  int oi = box_index32(o.ab, x0, y, z) + threadIdx.x;
+#pragma unroll 1
+  for (int x = x0 + threadIdx.x; x < xend; x += kEigRowThreads, p += kEigRowThreads, oi += kEigRowThreads) {
+    Sym3<float> s;
+    s.a = __ldg(p);
+    s.b = __ldg(p + ns);
+    s.c = __ldg(p + 2 * ns);
+    s.d = __ldg(p + 3 * ns);
+    s.e = __ldg(p + 4 * ns);
+    s.f = __ldg(p + 5 * ns);
+    float l[3], v[3];
+    if (!eig_closed(s, l, v, fb.gap))
+      push_fallback(fb, ((int64_t)blockIdx.z * ob.n[1] + blockIdx.y) * ob.n[0] + (x - ob.lo[0]));
+    write_voxel<VT, AT, FT, int, PLAIN>(o, oi, true, F, x, y, z, l, v, fill);
+  }
+}
+
 // The masked form: a CTA of kEigThreads threads takes kEigSpan consecutive
 // voxels of one row (voxel x0 + t + kEigThreads k for thread t, so that the
 // mask loads and the fill stores stay coalesced), writes the fill outputs of
@@ -369,6 +404,15 @@ cudaError_t launch_eig_angles(const float* S, const Box& sb, const Box& ob, cons
       } else {
         return launch_after(k_eig_angles_compact<-1, -1, -1, false>, gc, kEigThreads, 0, st, S, sb, ob, mask, mb, F, fill, o, mixed, fb);
       }
+    }
+    if (mask == nullptr && plain) {
+      const dim3 gr((ob.n[0] + kEigRowSpan - 1) / kEigRowSpan, ob.n[1], ob.n[2]);
+      if (o.vec_t == CT_OUT_F32 && o.ang_t == CT_OUT_F32 && o.fa_t == CT_OUT_F32)
+        return launch_after(k_eig_angles_rows<0, 0, 0, true>, gr, kEigRowThreads, 0, st, S, sb, ob, F, fill, o, fb);
+      if (o.vec_t == CT_OUT_F16 && o.ang_t == CT_OUT_F16 && o.fa_t == CT_OUT_F16)
+        return launch_after(k_eig_angles_rows<1, 1, 1, true>, gr, kEigRowThreads, 0, st, S, sb, ob, F, fill, o, fb);
+      if (o.vec_t == CT_OUT_F32 && o.ang_t == CT_OUT_U8Q && o.fa_t == CT_OUT_F16)
+        return launch_after(k_eig_angles_rows<0, 2, 1, true>, gr, kEigRowThreads, 0, st, S, sb, ob, F, fill, o, fb);
     }
     if (o.vec_t == CT_OUT_F32 && o.ang_t == CT_OUT_F32 && o.fa_t == CT_OUT_F32) {
       if (plain)

@@ -93,3 +93,21 @@ def test_tensor_core_rows_of_every_count(monkeypatch, ny, nz):
     S_o = O.structure_tensor(vol, sigma, rho)
     err = np.abs(S[:6 * n].reshape(S_o.shape) - S_o) / (S_o[0] + S_o[1] + S_o[2])[None]
     assert err.max() <= 2e-5, err.max()
+
+
+@pytest.mark.parametrize("nx", [5, 63, 65, 511, 512, 513, 1030])
+@pytest.mark.parametrize("types", [(_lib.CT_OUT_F32,) * 3, (_lib.CT_OUT_F16,) * 3,
+                                   (_lib.CT_OUT_F32, _lib.CT_OUT_U8Q, _lib.CT_OUT_F16)])
+def test_unmasked_eigen_rows_equal_the_masked_form(nx, types):
+    """Without a mask a CTA walks a span of one row; with a mask of ones each row segment's voxels
+    are listed first: the same arithmetic per voxel, so the same outputs to the bit, the
+    re-solved voxels of a flat slab among them."""
+    vol = _vol((5, 6, nx), nx)
+    vol[:, :, : nx // 4] = 1500
+    kw = dict(vec_type=types[0], angle_type=types[1], fa_type=types[2], raw=True)
+    cen, ax = (nx / 2 + 0.3, 2.0, 1.0), (0.1, 0.0, 1.0)
+    a = G.fused(vol, 1.0, 2.0, cen, ax, **kw)
+    b = G.fused(vol, 1.0, 2.0, cen, ax, mask=np.ones_like(vol, dtype=np.uint8), **kw)
+    for k in ("v", "ha", "ia", "fa"):
+        np.testing.assert_array_equal(a[k], b[k], err_msg=k)
+    assert a["stats"]["fallback_voxels"] == b["stats"]["fallback_voxels"]
