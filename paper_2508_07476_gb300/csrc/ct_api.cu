@@ -474,9 +474,11 @@ bool use_tc(const ct_plan P, const Scale& sc, const int dims[3], int axis) {
 // every row of every intermediate starts on a 32-byte sector and is read with
 // 16-byte copies whatever the volume's width (a ragged one otherwise goes
 // element by element through the rho passes: a 173 x 141 x 118 crop at R = 16, rho
-// x/y 118 and z 47 us, 90 and 33 us padded and with the CTA widths to fit).  The columns added lie beyond what any output reads; they hold
-// values of clamped coordinates.  Not for narrow boxes, where the padding would be a
-// large share, nor where it would push the planes past 32-bit indices.
+// x/y 118 and z 47 us, 90 and 33 us padded and with the CTA widths to fit).  The
+// columns added lie beyond what any output reads; they hold values of clamped
+// coordinates.  Not for narrow boxes, where the padding would be a large share, nor
+// where it would push the planes past 32-bit indices, nor where the device has no
+// room for it (chain_scratch).
 constexpr int kPadX = 8, kPadMinX = 64;
 
 struct ChainBoxes {
@@ -486,14 +488,14 @@ struct ChainBoxes {
   int64_t need;  // voxels per scratch buffer
 };
 
-ChainBoxes chain_boxes(const Scale& sc, const int dims[3], const Box& vb, const Box& ob) {
+ChainBoxes chain_boxes(const Scale& sc, const int dims[3], const Box& vb, const Box& ob, bool pad) {
   ChainBoxes c;
   c.G = grow_clip3(ob, sc.rr, dims);
   c.S = ob;
   Box g = c.G;
   g.lo[0] = g.lo[0] / kPadX * kPadX;
   g.n[0] = (c.G.lo[0] + c.G.n[0] - g.lo[0] + kPadX - 1) / kPadX * kPadX;
-  if (ob.n[0] >= kPadMinX && 6 * box_vox(g) < (int64_t(1) << 31) &&
+  if (pad && ob.n[0] >= kPadMinX && 6 * box_vox(g) < (int64_t(1) << 31) &&
       box_vox(grad_partial_box(g, vb, sc.rks, dims[2])) < (int64_t(1) << 31)) {
     c.G = g;
     c.S.n[0] = (ob.n[0] + kPadX - 1) / kPadX * kPadX;
@@ -504,6 +506,24 @@ ChainBoxes chain_boxes(const Scale& sc, const int dims[3], const Box& vb, const 
   return c;
 }
 
+// The chain's boxes with the slot's scratch sized for them: padded, or plain where the
+// padded scratch cannot be had (no room, or a stream that captures while the slot holds
+// less), so that padding fails no call that passes without it.
+ct_status chain_scratch(ct_plan P, const Scale& sc, const int dims[3], const Box& vb, const Box& ob, int slot,
+                        cudaStream_t st, ChainBoxes* cb) {
+  *cb = chain_boxes(sc, dims, vb, ob, true);
+  if (std::min(P->buf_cap[slot], P->fb_cap[slot]) >= cb->need) return ensure_scratch(P, slot, cb->need);
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  CT_CUDA(cudaStreamIsCapturing(st, &cap), "stream capture query");
+  if (cap == cudaStreamCaptureStatusNone) {
+    const ct_status rc = ensure_scratch(P, slot, cb->need);
+    if (rc != CT_ERR_OOM) return rc;
+    cudaGetLastError();  // the refused allocation is answered by the smaller one
+  }
+  *cb = chain_boxes(sc, dims, vb, ob, false);
+  return ensure_scratch(P, slot, cb->need);
+}
+
 Queue queue_of(ct_plan P, const Box& ob, cudaStream_t st) {
   return Queue(st, box_vox(ob) <= kEarlyMaxVox && !P->capturing);
 }
@@ -511,13 +531,13 @@ Queue queue_of(ct_plan P, const Box& ob, cudaStream_t st) {
 ct_status smooth_chain(ct_plan P, const Scale& sc, const int dims[3], const uint16_t* vol, const Box& vb,
                        const Box& ob, int slot, bool mixed, cudaStream_t st, int* zero, float* S_out, float** S_res,
                        Box* S_box) {
-  const ChainBoxes cb = chain_boxes(sc, dims, vb, ob);
+  ChainBoxes cb;
+  ct_status rc = chain_scratch(P, sc, dims, vb, ob, slot, st, &cb);
+  if (rc) return rc;
   const Box &G = cb.G, &Ab = cb.Ab;
   const Queue q = queue_of(P, ob, st);
   const Box So = S_out ? ob : cb.S;  // a caller's tensor is dense
   *S_box = So;
-  ct_status rc = ensure_scratch(P, slot, cb.need);
-  if (rc) return rc;
   float* A = P->buf[slot][0];
   float* B = P->buf[slot][1];
   const auto* tuning = tuned(P, sc, dims);
@@ -1490,16 +1510,25 @@ ct_status run_device_batch(ct_plan P, const ct_item* items, int n, cudaStream_t 
   const int k0 = pers.empty() || K == 1 ? 0 : 1;  // first stream of the per-item launches
   const int kn = std::max(1, K - k0);
   // scratch of every slot sized for its largest item, before any capture
-  std::vector<int64_t> gmax(K, 0);
+  // (padded where there is room for it: chain_scratch)
+  std::vector<int64_t> gmax(K, 0), gmin(K, 0);
   int64_t total = 0;
   for (int i = 0; i < n; ++i) total += box_vox(ctx[i].whole);
   for (size_t r = 0; r < rest.size(); ++r) {
     const int i = rest[r], k = k0 + (int)(r % kn);
-    gmax[k] = std::max(gmax[k], chain_boxes(ctx[i].sc, ctx[i].dims, ctx[i].whole, ctx[i].whole).need);
+    const auto need = [&](bool pad) {
+      return chain_boxes(ctx[i].sc, ctx[i].dims, ctx[i].whole, ctx[i].whole, pad).need;
+    };
+    gmax[k] = std::max(gmax[k], need(true));
+    gmin[k] = std::max(gmin[k], need(false));
   }
   for (int k = 0; k < K; ++k) {
     if ((rc = ensure_stream(P, k))) return rc;
-    if (gmax[k] > 0 && (rc = ensure_scratch(P, k, gmax[k]))) return rc;
+    if (gmax[k] > 0 && (rc = ensure_scratch(P, k, gmax[k])) == CT_ERR_OOM) {
+      cudaGetLastError();
+      rc = ensure_scratch(P, k, gmin[k]);
+    }
+    if (rc) return rc;
   }
   for (int k = 0; k < K && !pers.empty(); ++k)
     if (!P->wev[k]) CT_CUDA(cudaEventCreateWithFlags(&P->wev[k], cudaEventDisableTiming), "event creation");

@@ -111,3 +111,42 @@ def test_unmasked_eigen_rows_equal_the_masked_form(nx, types):
     for k in ("v", "ha", "ia", "fa"):
         np.testing.assert_array_equal(a[k], b[k], err_msg=k)
     assert a["stats"]["fallback_voxels"] == b["stats"]["fallback_voxels"]
+
+
+@pytest.mark.parametrize("first", [(65, 60, 50), (63, 62, 50)])
+def test_captured_box_equals_the_direct_call(first):
+    """A 65 x 60 x 50 box recorded into the caller's graph after a call that left scratch for
+    padded rows (the same box), and after one that left room for plain rows only (a narrower,
+    larger one): both replay to the direct call's outputs."""
+    nx, ny, nz = 160, 90, 80
+    vol = G.dev_u16(_vol((nz, ny, nx), 3))
+    params = _lib.make_params(1.0, 3.0, (300.0, 260.0, 10.0), (0.1, 0.1, 1.0), _lib.CT_PREC_MIXED)
+
+    def out(n):
+        return [torch.empty((k,) * (k > 1) + (n[2], n[1], n[0]), device="cuda") for k in (3, 1, 1, 1)]
+
+    def run(plan, n, o):
+        _lib.ct_run_box(plan, vol, (0, 0, 0), (nx, ny, nz), (3, 2, 1), n, None, *o)
+
+    box, plans = (65, 60, 50), [_lib.ct_plan_create(params, (nx, ny, nz)) for _ in range(2)]
+    st, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    try:
+        direct, warm, got = out(box), out(first), out(box)
+        run(plans[0], box, direct)
+        torch.cuda.synchronize()
+        with torch.cuda.stream(st):
+            run(plans[1], first, warm)
+        torch.cuda.synchronize()
+        with torch.cuda.graph(graph, stream=st):
+            run(plans[1], box, got)
+        for t in got:
+            t.fill_(-9.0)
+        for _ in range(2):
+            graph.replay()
+        torch.cuda.synchronize()
+        for a, b in zip(got, direct):
+            np.testing.assert_array_equal(a.cpu().numpy(), b.cpu().numpy())
+    finally:
+        del graph
+        for p in plans:
+            _lib.ct_plan_destroy(p)
