@@ -389,23 +389,30 @@ cudaError_t launch_eig_angles(const float* S, const Box& sb, const Box& ob, cons
       dim3 gc((ob.n[0] + kEigSpan - 1) / kEigSpan, ob.n[1], ob.n[2]);
       if (o.vec_t == CT_OUT_F32 && o.ang_t == CT_OUT_F32 && o.fa_t == CT_OUT_F32) {
         if (plain)
-          return launch_after(k_eig_angles_compact<0, 0, 0, true>, gc, kEigThreads, 0, st, S, sb, ob, mask, mb, F, fill, o, mixed, fb);
+          return launch_after(k_eig_angles_compact<0, 0, 0, true>, gc, kEigThreads, 0, st, S, sb, ob, mask, mb, F, fill, o, mixed,
+                              fb);
         else
-          return launch_after(k_eig_angles_compact<0, 0, 0, false>, gc, kEigThreads, 0, st, S, sb, ob, mask, mb, F, fill, o, mixed, fb);
+          return launch_after(k_eig_angles_compact<0, 0, 0, false>, gc, kEigThreads, 0, st, S, sb, ob, mask, mb, F, fill, o, mixed,
+                              fb);
       } else if (o.vec_t == CT_OUT_F16 && o.ang_t == CT_OUT_F16 && o.fa_t == CT_OUT_F16) {
         if (plain)
-          return launch_after(k_eig_angles_compact<1, 1, 1, true>, gc, kEigThreads, 0, st, S, sb, ob, mask, mb, F, fill, o, mixed, fb);
+          return launch_after(k_eig_angles_compact<1, 1, 1, true>, gc, kEigThreads, 0, st, S, sb, ob, mask, mb, F, fill, o, mixed,
+                              fb);
         else
-          return launch_after(k_eig_angles_compact<1, 1, 1, false>, gc, kEigThreads, 0, st, S, sb, ob, mask, mb, F, fill, o, mixed, fb);
+          return launch_after(k_eig_angles_compact<1, 1, 1, false>, gc, kEigThreads, 0, st, S, sb, ob, mask, mb, F, fill, o, mixed,
+                              fb);
       } else if (o.vec_t == CT_OUT_F32 && o.ang_t == CT_OUT_U8Q && o.fa_t == CT_OUT_F16 && plain) {
-        return launch_after(k_eig_angles_compact<0, 2, 1, true>, gc, kEigThreads, 0, st, S, sb, ob, mask, mb, F, fill, o, mixed, fb);
+        return launch_after(k_eig_angles_compact<0, 2, 1, true>, gc, kEigThreads, 0, st, S, sb, ob, mask, mb, F, fill, o, mixed,
+                            fb);
       } else if (o.ang_t == CT_OUT_U8Q && o.fa_t == CT_OUT_F16) {
-        return launch_after(k_eig_angles_compact<-1, 2, 1, false>, gc, kEigThreads, 0, st, S, sb, ob, mask, mb, F, fill, o, mixed, fb);
+        return launch_after(k_eig_angles_compact<-1, 2, 1, false>, gc, kEigThreads, 0, st, S, sb, ob, mask, mb, F, fill, o, mixed,
+                            fb);
       } else {
-        return launch_after(k_eig_angles_compact<-1, -1, -1, false>, gc, kEigThreads, 0, st, S, sb, ob, mask, mb, F, fill, o, mixed, fb);
+        return launch_after(k_eig_angles_compact<-1, -1, -1, false>, gc, kEigThreads, 0, st, S, sb, ob, mask, mb, F, fill, o, mixed,
+                            fb);
       }
     }
-    if (mask == nullptr && plain) {
+    if (mask == nullptr && plain) {  // k_eig_angles_rows has both forms' times
       const dim3 gr((ob.n[0] + kEigRowSpan - 1) / kEigRowSpan, ob.n[1], ob.n[2]);
       if (o.vec_t == CT_OUT_F32 && o.ang_t == CT_OUT_F32 && o.fa_t == CT_OUT_F32)
         return launch_after(k_eig_angles_rows<0, 0, 0, true>, gr, kEigRowThreads, 0, st, S, sb, ob, F, fill, o, fb);
@@ -431,7 +438,6 @@ cudaError_t launch_eig_angles(const float* S, const Box& sb, const Box& ob, cons
     } else {
       return launch_after(k_eig_angles32<-1, -1, -1, false>, g3, nt, 0, st, S, sb, ob, mask, mb, F, fill, o, mixed, fb);
     }
-    return cudaGetLastError();
   }
   // the encodings of the common configurations are compiled in; others are read at run time
   if (o.vec_t == CT_OUT_F32 && o.ang_t == CT_OUT_F32 && o.fa_t == CT_OUT_F32)
@@ -442,7 +448,6 @@ cudaError_t launch_eig_angles(const float* S, const Box& sb, const Box& ob, cons
     return launch_after(k_eig_angles<-1, 2, 1>, grid, nt, 0, st, S, sb, ob, mask, mb, F, fill, o, mixed, fb);
   else
     return launch_after(k_eig_angles<-1, -1, -1>, grid, nt, 0, st, S, sb, ob, mask, mb, F, fill, o, mixed, fb);
-  return cudaGetLastError();
 }
 
 cudaError_t launch_eig_angles_fallback(const float* S, const Box& sb, const Box& ob, const uint8_t* mask,

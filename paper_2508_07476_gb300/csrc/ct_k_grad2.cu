@@ -11,8 +11,8 @@
 // partial fields cross HBM once (12 B written and read per voxel), as a plane of
 // (F0, F1) pairs and a plane of F2: two stores and two copies per voxel
 // instead of three of each, and the pairs are what the z pass's packed
-// arithmetic takes (512^3: x/y
-// 604 -> 615 us, z 500 -> 433 us).
+// arithmetic takes (512^3: x/y 604 -> 615 us, z 500 -> 433 us; x/y 576 us with the
+// slots below).
 //
 // Every pass folds the +k / -k taps (sums for the smoothing taps w,
 // differences for the derivative taps c), so a constant volume gives an

@@ -6,10 +6,14 @@
 //    memory; each thread computes 8 consecutive outputs of one row from a
 //    register window filled by 16-byte shared loads (one load per 28 FMAs at
 //    R = 24).  Results leave through shared memory as coalesced stores.
-//  * y and z passes: one thread per (column, component) walks the pass axis
-//    with a register window of the last 2R+1 inputs plus D prefetched ones;
-//    each step costs one coalesced load, 2R+1 FMAs and one coalesced store, and
-//    no halo is re-read except at segment starts.
+//  * z pass (k_rho_z2): one thread per pair of neighbouring columns and
+//    component walks z in blocks of 8 outputs, with a register window of the
+//    block's inputs and the 2R before them, the next two blocks in flight.
+//  * y pass alone, and z over rows of odd length (k_rho_stream): one thread per
+//    (column, component) walks the pass axis with a register window of the
+//    last 2R+1 inputs plus D prefetched ones; each step costs one coalesced
+//    load, 2R+1 FMAs and one coalesced store.  No halo is re-read in either
+//    except at segment starts.
 #include "ct_common.cuh"
 #include "ct_launch.h"
 

@@ -54,13 +54,14 @@ cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, size_t sme
 // resident at once on `sms` SMs.  The cheapest of up to 64 cuts, whole waves
 // of CTAs counted as they run side by side, the last one by the square root of
 // the share of an SM's CTAs it still holds (fewer CTAs run faster, but not in
-// proportion) and no less than kLoneCta (one waits for its own loads and barriers).  seg: a multiple of unit.  Before, the walks were
-// cut by powers of two while the grid was below a fixed size and a segment
-// above a fixed length, so a 64^3 volume ran grad_z in 16 CTAs: its gradient
-// x/y, z and rho z passes 15.4, 16.4, 10.4 us, and 10.8, 8.3, 8.1 now;
-// 173 x 141 x 118: gradient 39.8 + 37.6 us, and 25.8 + 20.5 now.  The times are
-// flat in the weights: kLoneCta 0.25 .. 0.8 and warm x 0.6 .. 1.5 move none of the
-// measured volumes by more than 1%.
+// proportion) and no less than kLoneCta (one waits for its own loads and
+// barriers).  seg: a multiple of unit.  Before, the walks were cut by powers of
+// two while the grid was below a fixed size and a segment above a fixed length,
+// so a 64^3 volume ran grad_z in 16 CTAs: its gradient x/y, z and rho z passes
+// 15.4, 16.4, 10.4 us, and 10.8, 8.3, 8.1 so; 173 x 141 x 118: gradient
+// 39.8 + 37.6 us, and 25.8 + 18.5.  The times are flat in the weights: kLoneCta
+// 0.25 .. 0.8 and warm x 0.6 .. 1.5 move none of the measured volumes by more
+// than 1%.
 constexpr double kLoneCta = 0.5;
 inline int walk_segment(int64_t ctas, int n, int unit, double warm, int slots, int sms) {
   double best = 1e300;
