@@ -150,3 +150,40 @@ def test_captured_box_equals_the_direct_call(first):
         del graph
         for p in plans:
             _lib.ct_plan_destroy(p)
+
+
+@pytest.mark.parametrize("chunk", [(0, 0, 9), (0, 0, 16), (0, 0, 64), (0, 0, 149), (72, 0, 20), (72, 60, 33)])
+@pytest.mark.parametrize("masked", [False, True])
+def test_host_slabs_of_every_count_equal_the_device_call(chunk, masked):
+    """Two host items of one call, in slabs of which each reuses its buffers two slabs later
+    while the copies of others are in flight: both equal the call on device memory."""
+    rng = np.random.default_rng(8)
+    dims = [(200, 130, 150), (96, 70, 41)]
+    vols = [_vol(d[::-1], 11 + k) for k, d in enumerate(dims)]
+    masks = [(rng.random(d[::-1]) < 0.7).astype(np.uint8) if masked else None for d in dims]
+    params = _lib.make_params(1.0, 3.0, (300.0, 260.0, 10.0), (0.1, 0.1, 1.0), _lib.CT_PREC_MIXED,
+                              chunk=chunk)
+
+    def run(on_host):
+        outs, items, keep = [], [], []
+        plan = _lib.ct_plan_create(params, dims[0])
+        for (nx, ny, nz), vol, mask in zip(dims, vols, masks):
+            v = torch.from_numpy(vol.view(np.int16))
+            m = None if mask is None else torch.from_numpy(mask)
+            kw = dict(pin_memory=True) if on_host else dict(device="cuda")
+            v, m = [None if t is None else t.pin_memory() if on_host else t.cuda() for t in (v, m)]
+            o = [torch.full((k,) * (k > 1) + (nz, ny, nx), -9.0, **kw) for k in (3, 1, 1, 1)]
+            items.append(_lib.make_item(v, (nx, ny, nz), m, *o))
+            outs.append(o)
+            keep += [v, m]
+        try:
+            for _ in range(2 if on_host else 1):
+                _lib.ct_run_chunks(plan, items, on_host)
+            torch.cuda.synchronize()
+        finally:
+            _lib.ct_plan_destroy(plan)
+        return outs
+
+    for a, b in zip(run(True), run(False)):
+        for p, q in zip(a, b):
+            np.testing.assert_array_equal(p.numpy(), q.cpu().numpy())
