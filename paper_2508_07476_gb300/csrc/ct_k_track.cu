@@ -52,7 +52,9 @@ __device__ __forceinline__ float weight(const Cell& c, int k) {
 // FA), all of them in flight together.  The tracks of a warp lie anywhere in
 // the volume, so every load is its own sector: the kernel is bound by the
 // number of those (512^3, 200 000 seeds, 200 steps of 0.5:
-// 118.8 ms with the values read again at every evaluation, 19.3 ms held).
+// 118.8 ms with the values read again at every evaluation, 19.1 ms held, 89 GB
+// of sectors from DRAM; a cell's x neighbours as one aligned 8- or 16-byte
+// load beside a predicated 4-byte one: 21.8, 30.1 ms).
 struct Field {
   const float* __restrict__ vec;
   const float* __restrict__ fa;  // or nullptr
