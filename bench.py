@@ -412,7 +412,7 @@ def _kernel_algorithmic(name: str, nvox: int, rs: int, rr: int, inside: float = 
 MEASURED_TRAFFIC = {"rho_x_tc": (45.1, "profiles/kernels_annulus256.md"),
                     "rho_y_tc": (44.8, "profiles/kernels_annulus256.md"),
                     "rho_z_tc_g16": (26.6, "profiles/kernels_annulus256.md"),
-                    "grad_z_g16": (16.4, "profiles/kernels_annulus256.md"),
+                    "grad_z_g16": (16.2, "profiles/kernels_annulus256.md"),
                     "grad_xy": (10.4, "profiles/kernels_annulus256.md"),
                     "eig_angles": (36.4, "profiles/kernels_annulus256.md")}
 
