@@ -159,6 +159,7 @@ struct ct_plan_s {
   unsigned long long* fb_total = nullptr;  // running count of re-solved voxels
   int64_t* fb_list[kSlots] = {};
   int64_t fb_cap[kSlots] = {};
+  uint64_t scratch_gen[kSlots] = {};  // counts the slot's replaced buffers (buf, fb_list): a graph holds their addresses
   // device word counting the tensor-core CTAs of this plan that gave up a
   // bounded wait (read and cleared by ct_plan_sync)
   unsigned int* d_timeouts = nullptr;
@@ -320,6 +321,7 @@ ct_status ensure_fallback(ct_plan P, int slot, int64_t vox) {
     CT_CUDA(cudaMemset(P->fb_total, 0, sizeof(unsigned long long)), "counter reset");
   }
   if (P->fb_cap[slot] < vox) {
+    ++P->scratch_gen[slot];
     if (P->fb_list[slot]) cudaFree(P->fb_list[slot]);
     P->fb_list[slot] = nullptr;
     P->fb_cap[slot] = 0;
@@ -331,6 +333,7 @@ ct_status ensure_fallback(ct_plan P, int slot, int64_t vox) {
 
 ct_status ensure_scratch(ct_plan P, int slot, int64_t vox) {
   if (P->buf_cap[slot] < vox) {
+    ++P->scratch_gen[slot];
     for (int k = 0; k < 2; ++k) {
       if (P->buf[slot][k]) cudaFree(P->buf[slot][k]);
       P->buf[slot][k] = nullptr;
@@ -1467,9 +1470,9 @@ ct_status run_persistent_waves(ct_plan P, const std::vector<WaveRec>& waves, int
 // frames): items go round-robin onto up to kSlots streams, each with its own
 // scratch slot, so that small volumes run side by side.  The whole
 // multi-stream launch sequence is captured once into a CUDA graph (cached
-// under a hash of the item list and the plan's settings) and replayed with a
-// single graph launch; with graphs off, every item is launched in turn on the
-// caller's stream.
+// under a hash of the item list, the plan's settings and the generations of the
+// slots' scratch, whose addresses it holds) and replayed with a single graph
+// launch; with graphs off, every item is launched in turn on the caller's stream.
 ct_status run_device_batch(ct_plan P, const ct_item* items, int n, cudaStream_t user) {
   bool mixed = P->p.precision == CT_PREC_MIXED;
   std::vector<ItemCtx> ctx(n);
@@ -1586,6 +1589,7 @@ ct_status run_device_batch(ct_plan P, const ct_item* items, int n, cudaStream_t 
   key = fnv1a(key, &K, sizeof K);
   key = fnv1a(key, &P->batch_persistent, sizeof P->batch_persistent);
   key = fnv1a(key, &P->batch_bytes, sizeof P->batch_bytes);
+  key = fnv1a(key, P->scratch_gen, sizeof P->scratch_gen[0] * (size_t)K);  // (every slot's scratch is in place)
   if (!P->graph_exec || P->graph_key != key) {
     if (P->graph_exec) cudaGraphExecDestroy(P->graph_exec);
     if (P->graph) cudaGraphDestroy(P->graph);
