@@ -331,7 +331,7 @@ ct_status ensure_fallback(ct_plan P, int slot, int64_t vox) {
   return CT_OK;
 }
 
-ct_status ensure_scratch(ct_plan P, int slot, int64_t vox) {
+ct_status ensure_buffers(ct_plan P, int slot, int64_t vox) {
   if (P->buf_cap[slot] < vox) {
     ++P->scratch_gen[slot];
     for (int k = 0; k < 2; ++k) {
@@ -342,7 +342,12 @@ ct_status ensure_scratch(ct_plan P, int slot, int64_t vox) {
     for (int k = 0; k < 2; ++k) CT_CUDA(cudaMalloc(&P->buf[slot][k], sizeof(float) * 6 * vox), "scratch allocation");
     P->buf_cap[slot] = vox;
   }
-  return ensure_fallback(P, slot, vox);
+  return CT_OK;
+}
+
+ct_status ensure_scratch(ct_plan P, int slot, int64_t vox) {
+  const ct_status rc = ensure_buffers(P, slot, vox);
+  return rc ? rc : ensure_fallback(P, slot, vox);
 }
 
 Fallback fallback_of(ct_plan P, int slot) {
@@ -480,8 +485,8 @@ bool use_tc(const ct_plan P, const Scale& sc, const int dims[3], int axis) {
 // x/y 118 and z 47 us, 90 and 33 us padded and with the CTA widths to fit).  The
 // columns added lie beyond what any output reads; they hold values of clamped
 // coordinates.  Not for narrow boxes, where the padding would be a large share, nor
-// where it would push the planes past 32-bit indices, nor where the device has no
-// room for it (chain_scratch).
+// where it would push the planes past 32-bit indices, nor where the slot's scratch does
+// not hold it (ensure_chain_scratch).
 constexpr int kPadX = 8, kPadMinX = 64;
 
 struct ChainBoxes {
@@ -509,22 +514,30 @@ ChainBoxes chain_boxes(const Scale& sc, const int dims[3], const Box& vb, const 
   return c;
 }
 
-// The chain's boxes with the slot's scratch sized for them: padded, or plain where the
-// padded scratch cannot be had (no room, or a stream that captures while the slot holds
-// less), so that padding fails no call that passes without it.
-ct_status chain_scratch(ct_plan P, const Scale& sc, const int dims[3], const Box& vb, const Box& ob, int slot,
-                        cudaStream_t st, ChainBoxes* cb) {
-  *cb = chain_boxes(sc, dims, vb, ob, true);
-  if (std::min(P->buf_cap[slot], P->fb_cap[slot]) >= cb->need) return ensure_scratch(P, slot, cb->need);
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  CT_CUDA(cudaStreamIsCapturing(st, &cap), "stream capture query");
-  if (cap == cudaStreamCaptureStatusNone) {
-    const ct_status rc = ensure_scratch(P, slot, cb->need);
-    if (rc != CT_ERR_OOM) return rc;
-    cudaGetLastError();  // the refused allocation is answered by the smaller one
+// Scratch of a slot for a chain of `plain` voxels per buffer, or `padded` with padded
+// rows.  Buffers are replaced only where the plain rows do not fit: by padded ones, or by plain
+// ones where those are refused.  Buffers that hold the plain rows stay, so that padding
+// replaces nothing that a call without it would keep: a caller's own graph may hold their
+// addresses, and a device that refused the padded size once is not asked on every call.
+ct_status ensure_chain_scratch(ct_plan P, int slot, int64_t plain, int64_t padded) {
+  if (P->buf_cap[slot] < plain) {
+    const ct_status rc = ensure_buffers(P, slot, padded);
+    if (rc == CT_ERR_OOM && padded > plain)
+      cudaGetLastError();  // the refused allocation is answered by the smaller one
+    else if (rc)
+      return rc;
   }
-  *cb = chain_boxes(sc, dims, vb, ob, false);
-  return ensure_scratch(P, slot, cb->need);
+  return ensure_scratch(P, slot, plain);
+}
+
+// The chain's boxes with the slot's scratch in place: padded where its buffers hold that.
+ct_status chain_scratch(ct_plan P, const Scale& sc, const int dims[3], const Box& vb, const Box& ob, int slot,
+                        ChainBoxes* cb) {
+  const ChainBoxes plain = chain_boxes(sc, dims, vb, ob, false);
+  *cb = chain_boxes(sc, dims, vb, ob, true);
+  const ct_status rc = ensure_chain_scratch(P, slot, plain.need, cb->need);
+  if (rc == CT_OK && P->buf_cap[slot] < cb->need) *cb = plain;
+  return rc;
 }
 
 Queue queue_of(ct_plan P, const Box& ob, cudaStream_t st) {
@@ -535,7 +548,7 @@ ct_status smooth_chain(ct_plan P, const Scale& sc, const int dims[3], const uint
                        const Box& ob, int slot, bool mixed, cudaStream_t st, int* zero, float* S_out, float** S_res,
                        Box* S_box) {
   ChainBoxes cb;
-  ct_status rc = chain_scratch(P, sc, dims, vb, ob, slot, st, &cb);
+  ct_status rc = chain_scratch(P, sc, dims, vb, ob, slot, &cb);
   if (rc) return rc;
   const Box &G = cb.G, &Ab = cb.Ab;
   const Queue q = queue_of(P, ob, st);
@@ -1513,7 +1526,6 @@ ct_status run_device_batch(ct_plan P, const ct_item* items, int n, cudaStream_t 
   const int k0 = pers.empty() || K == 1 ? 0 : 1;  // first stream of the per-item launches
   const int kn = std::max(1, K - k0);
   // scratch of every slot sized for its largest item, before any capture
-  // (padded where there is room for it: chain_scratch)
   std::vector<int64_t> gmax(K, 0), gmin(K, 0);
   int64_t total = 0;
   for (int i = 0; i < n; ++i) total += box_vox(ctx[i].whole);
@@ -1527,11 +1539,7 @@ ct_status run_device_batch(ct_plan P, const ct_item* items, int n, cudaStream_t 
   }
   for (int k = 0; k < K; ++k) {
     if ((rc = ensure_stream(P, k))) return rc;
-    if (gmax[k] > 0 && (rc = ensure_scratch(P, k, gmax[k])) == CT_ERR_OOM) {
-      cudaGetLastError();
-      rc = ensure_scratch(P, k, gmin[k]);
-    }
-    if (rc) return rc;
+    if (gmax[k] > 0 && (rc = ensure_chain_scratch(P, k, gmin[k], gmax[k]))) return rc;
   }
   for (int k = 0; k < K && !pers.empty(); ++k)
     if (!P->wev[k]) CT_CUDA(cudaEventCreateWithFlags(&P->wev[k], cudaEventDisableTiming), "event creation");

@@ -66,3 +66,37 @@ def test_equal_batches_around_calls_that_replace_the_scratch():
         assert all(bool((t == 3.0).all()) for t in others)
     finally:
         _lib.ct_plan_destroy(plan)
+
+
+def test_a_recorded_box_after_the_same_direct_call():
+    """A 66 x 60 x 50 box recorded into the caller's graph on scratch that a narrower box left (it holds
+    the plain rows but not the padded ones), then called directly on the same plan: the direct
+    call leaves the recorded scratch in place, and the graph replays to its outputs."""
+    vol = G.dev_u16(_vol(DIMS[::-1], 3))
+    params = _lib.make_params(**PARAMS)
+
+    def run(plan, n, o):
+        _lib.ct_run_box(plan, vol, (0, 0, 0), DIMS, (3, 2, 1), n, None, *o)
+
+    first, box, plans = (63, 68, 50), (66, 60, 50), [_lib.ct_plan_create(params, DIMS) for _ in range(2)]
+    st, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    try:
+        padded, warm, got, plain = _out(box), _out(first), _out(box), _out(box)
+        run(plans[0], box, padded)
+        torch.cuda.synchronize()
+        with torch.cuda.stream(st):
+            run(plans[1], first, warm)
+        torch.cuda.synchronize()
+        with torch.cuda.graph(graph, stream=st):
+            run(plans[1], box, got)
+        run(plans[1], box, plain)
+        torch.cuda.synchronize()
+        graph.replay()
+        torch.cuda.synchronize()
+        for a, b, c in zip(got, plain, padded):
+            np.testing.assert_array_equal(a.cpu().numpy(), c.cpu().numpy())
+            np.testing.assert_array_equal(b.cpu().numpy(), c.cpu().numpy())
+    finally:
+        del graph
+        for p in plans:
+            _lib.ct_plan_destroy(p)

@@ -92,3 +92,50 @@ def test_a_batch_graph_is_recorded_anew_when_its_scratch_has_moved(plan, grow):
     end = plan.counts()
     assert end[STALE] == before[STALE]
     assert end[INSTANTIATED] - moved[INSTANTIATED] == 1 and end[LAUNCHED] - moved[LAUNCHED] == 2
+
+
+NARROW, WIDE = (63, 68, 50), (66, 60, 50)  # the narrow box's scratch holds the wide one's rows, but not padded
+
+
+def test_padding_does_not_move_scratch_that_holds_the_plain_rows(plan):
+    """The wide box recorded by the caller on the narrow one's scratch, then called directly: the
+    buffers whose addresses the record holds stay."""
+    plan.box(NARROW)
+    before = plan.counts()
+    plan.lib.double_user_capture(1)
+    plan.box(WIDE)
+    plan.lib.double_user_capture(0)
+    plan.box(WIDE)
+    assert plan.counts() == before
+
+
+def refuse_padding(plan, call):
+    """The smallest limit on a block under which a first `call` passes (its plain rows), above that
+    of the re-solve lists; a smaller one refuses it."""
+    lo, hi = 0, 1 << 40
+    while hi - lo > 1:
+        mid = (lo + hi) // 2
+        plan.lib.double_limit(mid)
+        probe = Plan(plan.lib, plan.dims)
+        try:
+            call(probe)
+            hi = mid
+        except AssertionError:
+            lo = mid
+        finally:
+            plan.lib.ct_plan_destroy(probe.p)
+    plan.lib.double_limit(hi)
+
+
+@pytest.mark.parametrize("call", [lambda p: p.box(WIDE), lambda p: p.batch(BATCH)], ids=["box", "batch"])
+def test_a_refused_padding_is_not_asked_for_again(plan, call):
+    """Where the padded scratch is refused a call takes plain rows; the next equal call allocates
+    and frees nothing, nor does one after the device has room again."""
+    refuse_padding(plan, call)
+    call(plan)
+    before = plan.counts()
+    call(plan)
+    assert plan.counts()[:3] == before[:3]
+    plan.lib.double_limit(ctypes.c_uint64(-1).value)
+    call(plan)
+    assert plan.counts()[:3] == before[:3] and plan.counts()[STALE] == before[STALE]
