@@ -545,12 +545,15 @@ Queue queue_of(ct_plan P, const Box& ob, cudaStream_t st) {
 }
 
 ct_status smooth_chain(ct_plan P, const Scale& sc, const int dims[3], const uint16_t* vol, const Box& vb,
-                       const Box& ob, int slot, bool mixed, cudaStream_t st, int* zero, float* S_out, float** S_res,
+                       const Box& ob, int slot, bool mixed, cudaStream_t st, bool eig, float* S_out, float** S_res,
                        Box* S_box) {
   ChainBoxes cb;
   ct_status rc = chain_scratch(P, sc, dims, vb, ob, slot, &cb);
   if (rc) return rc;
   const Box &G = cb.G, &Ab = cb.Ab;
+  // the first kernel clears the re-solve counter of the eigen stage that follows (a
+  // memset between the kernels would keep the next one from starting early)
+  int* zero = eig ? P->fb_count[slot] : nullptr;
   const Queue q = queue_of(P, ob, st);
   const Box So = S_out ? ob : cb.S;  // a caller's tensor is dense
   *S_box = So;
@@ -625,7 +628,7 @@ ct_status tensor_stages(ct_plan P, const Scale& sc, const int dims[3], const uin
                         const Box& ob, float* S_out, int slot, bool mixed, cudaStream_t st) {
   float* S = nullptr;
   Box sb;
-  return smooth_chain(P, sc, dims, vol, vb, ob, slot, mixed, st, nullptr, S_out, &S, &sb);
+  return smooth_chain(P, sc, dims, vol, vb, ob, slot, mixed, st, false, S_out, &S, &sb);
 }
 
 ct_status eig_stage(ct_plan P, const float* S, const Box& sb, const Box& ob, const uint8_t* mask, const Box& mb, const Frame& F,
@@ -639,11 +642,7 @@ ct_status fused_stages(ct_plan P, const Scale& sc, const int dims[3], const uint
                        bool mixed, cudaStream_t st) {
   float* S = nullptr;
   Box sb;
-  ct_status rc = ensure_fallback(P, slot, box_vox(ob));
-  // the chain's first kernel clears the re-solve counter (a memset between the
-  // kernels would keep the next one from starting early)
-  if (rc == CT_OK)
-    rc = smooth_chain(P, sc, dims, vol, vb, ob, slot, mixed, st, P->fb_count[slot], nullptr, &S, &sb);
+  ct_status rc = smooth_chain(P, sc, dims, vol, vb, ob, slot, mixed, st, true, nullptr, &S, &sb);
   if (rc) return rc;
   const auto* t = tuned(P, sc, dims);
   return eig_stage(P, S, sb, ob, mask, mb, F, o, slot, mixed, t && t->eig_compact >= 0 ? t->eig_compact != 0 : P->eig_compact,

@@ -139,3 +139,11 @@ def test_a_refused_padding_is_not_asked_for_again(plan, call):
     plan.lib.double_limit(ctypes.c_uint64(-1).value)
     call(plan)
     assert plan.counts()[:3] == before[:3] and plan.counts()[STALE] == before[STALE]
+
+
+def test_a_first_call_allocates_its_scratch_once(plan):
+    """Two buffers, the re-solve list and its two counters, and nothing given back."""
+    before = plan.counts()
+    plan.box(WIDE)
+    after = plan.counts()
+    assert after[MALLOCS] - before[MALLOCS] == 5 and after[FREES] == before[FREES]
