@@ -48,10 +48,14 @@ __device__ __forceinline__ int clamp_to(int p, int dim, int lo, int n) {
   return clampi(clampi(p, 0, dim - 1), lo, lo + n - 1);
 }
 
-// First statement of the chain's kernels, which are launched so that their CTAs
-// may start while the previous kernel of the stream still runs (launch_after):
-// waits until that kernel has finished and its writes are visible, then lets
-// the next kernel's CTAs start.  Nothing of the kernel's work comes before it.
+// In the chain's kernels, which are launched so that their CTAs may start while the
+// previous kernel of the stream still runs (launch_after): waits until that kernel
+// has finished and its writes are visible, then lets the next kernel's CTAs
+// start.  No access to global memory comes before it (k_rho_tc sets up its shared and
+// tensor memory first: every CTA of a kernel has its tensor memory before the
+// next kernel's CTAs can ask for any).  What the previous kernel wrote is read by
+// plain loads (__ldca) or asynchronous copies, never by __ldg: that asks for data that
+// does not change while the kernel runs, and here it may run before the data is there.
 __device__ __forceinline__ void after_previous() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

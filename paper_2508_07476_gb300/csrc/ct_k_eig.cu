@@ -20,12 +20,12 @@ namespace ct {
 
 __device__ __forceinline__ Sym3<float> load_sym(const float* S, int64_t n, int64_t i) {
   Sym3<float> s;
-  s.a = __ldg(S + i);
-  s.b = __ldg(S + n + i);
-  s.c = __ldg(S + 2 * n + i);
-  s.d = __ldg(S + 3 * n + i);
-  s.e = __ldg(S + 4 * n + i);
-  s.f = __ldg(S + 5 * n + i);
+  s.a = __ldca(S + i);
+  s.b = __ldca(S + n + i);
+  s.c = __ldca(S + 2 * n + i);
+  s.d = __ldca(S + 3 * n + i);
+  s.e = __ldca(S + 4 * n + i);
+  s.f = __ldca(S + 5 * n + i);
   return s;
 }
 
@@ -131,12 +131,12 @@ __device__ __forceinline__ void eig32_body(const float* __restrict__ S, Box sb, 
     const int ns = sb.n[0] * sb.n[1] * sb.n[2];
     const int si = box_index32(sb, x, y, z);
     Sym3<float> s;
-    s.a = __ldg(S + si);
-    s.b = __ldg(S + ns + si);
-    s.c = __ldg(S + 2 * ns + si);
-    s.d = __ldg(S + 3 * ns + si);
-    s.e = __ldg(S + 4 * ns + si);
-    s.f = __ldg(S + 5 * ns + si);
+    s.a = __ldca(S + si);
+    s.b = __ldca(S + ns + si);
+    s.c = __ldca(S + 2 * ns + si);
+    s.d = __ldca(S + 3 * ns + si);
+    s.e = __ldca(S + 4 * ns + si);
+    s.f = __ldca(S + 5 * ns + si);
     if (!eig_closed(s, l, v, fb.gap))
       push_fallback(fb, ((int64_t)blk.z() * ob.n[1] + blk.y()) * ob.n[0] + (x - ob.lo[0]));
   }
@@ -174,12 +174,12 @@ __global__ void __launch_bounds__(kEigRowThreads, 24)
 #pragma unroll 1
   for (int x = x0 + threadIdx.x; x < xend; x += kEigRowThreads, p += kEigRowThreads, oi += kEigRowThreads) {
     Sym3<float> s;
-    s.a = __ldg(p);
-    s.b = __ldg(p + ns);
-    s.c = __ldg(p + 2 * ns);
-    s.d = __ldg(p + 3 * ns);
-    s.e = __ldg(p + 4 * ns);
-    s.f = __ldg(p + 5 * ns);
+    s.a = __ldca(p);
+    s.b = __ldca(p + ns);
+    s.c = __ldca(p + 2 * ns);
+    s.d = __ldca(p + 3 * ns);
+    s.e = __ldca(p + 4 * ns);
+    s.f = __ldca(p + 5 * ns);
     float l[3], v[3];
     if (!eig_closed(s, l, v, fb.gap))
       push_fallback(fb, ((int64_t)blockIdx.z * ob.n[1] + blockIdx.y) * ob.n[0] + (x - ob.lo[0]));
@@ -266,12 +266,12 @@ __device__ __forceinline__ void eig_compact_body(const float* __restrict__ S, Bo
       const int i = i0 + kEigThreads * u;
       xs[u] = x0 + list[i < total ? i : i0];
       const int si = box_index32(sb, xs[u], y, z);
-      s[u].a = __ldg(S + si);
-      s[u].b = __ldg(S + ns + si);
-      s[u].c = __ldg(S + 2 * ns + si);
-      s[u].d = __ldg(S + 3 * ns + si);
-      s[u].e = __ldg(S + 4 * ns + si);
-      s[u].f = __ldg(S + 5 * ns + si);
+      s[u].a = __ldca(S + si);
+      s[u].b = __ldca(S + ns + si);
+      s[u].c = __ldca(S + 2 * ns + si);
+      s[u].d = __ldca(S + 3 * ns + si);
+      s[u].e = __ldca(S + 4 * ns + si);
+      s[u].f = __ldca(S + 5 * ns + si);
     }
 #pragma unroll
     for (int u = 0; u < kEigIlp; ++u) {

@@ -121,11 +121,11 @@ __device__ __forceinline__ void grad_xy_body(const uint16_t* __restrict__ vol, c
       const int y = min(max(p0 - RS - G::PAD + b * TB + q_row[i], ylo), yhi);
       const uint16_t* row = plane + (int64_t)(y - vb.lo[1]) * vb.n[0] - vb.lo[0];
       if (q_fast[i]) {
-        pre[i] = __ldg(reinterpret_cast<const uint4*>(row + q_col[i]));
+        pre[i] = __ldca(reinterpret_cast<const uint4*>(row + q_col[i]));
       } else {
         uint32_t h[8];
 #pragma unroll
-        for (int e = 0; e < 8; ++e) h[e] = __ldg(row + clamp_to(q_col[i] + e, dimx, vb.lo[0], vb.n[0]));
+        for (int e = 0; e < 8; ++e) h[e] = __ldca(row + clamp_to(q_col[i] + e, dimx, vb.lo[0], vb.n[0]));
         pre[i] = make_uint4(h[0] | (h[1] << 16), h[2] | (h[3] << 16), h[4] | (h[5] << 16), h[6] | (h[7] << 16));
       }
     }
@@ -269,11 +269,11 @@ __global__ void __launch_bounds__(XT, 512 / XT)
         if (SLOTS)
           cp_async16_u16((uint32_t)__cvta_generic_to_shared(slot(b, i)), row + q_col[i]);
         else
-          pre[SLOTS ? 0 : i] = __ldg(reinterpret_cast<const uint4*>(row + q_col[i]));
+          pre[SLOTS ? 0 : i] = __ldca(reinterpret_cast<const uint4*>(row + q_col[i]));
       } else {
         uint32_t h[8];
 #pragma unroll
-        for (int e = 0; e < 8; ++e) h[e] = __ldg(row + clamp_to(q_col[i] + e, dimx, vb.lo[0], vb.n[0]));
+        for (int e = 0; e < 8; ++e) h[e] = __ldca(row + clamp_to(q_col[i] + e, dimx, vb.lo[0], vb.n[0]));
         const uint4 q = make_uint4(h[0] | (h[1] << 16), h[2] | (h[3] << 16), h[4] | (h[5] << 16), h[6] | (h[7] << 16));
         if (SLOTS)
           *slot(b, i) = q;

@@ -83,12 +83,12 @@ __global__ void __launch_bounds__(kRxThreads, CT_RX_MINB)
     const float* rowp = in + comp * nib + rin[row] - ib.lo[0];
     float4 v;
     if (gx0 >= xlo_ok && gx0 + 3 < xhi_ok && ((reinterpret_cast<uintptr_t>(rowp + gx0) & 15) == 0)) {
-      v = __ldg(reinterpret_cast<const float4*>(rowp + gx0));
+      v = __ldca(reinterpret_cast<const float4*>(rowp + gx0));
     } else {
-      v.x = __ldg(rowp + clamp_to(gx0, dimx, ib.lo[0], ib.n[0]));
-      v.y = __ldg(rowp + clamp_to(gx0 + 1, dimx, ib.lo[0], ib.n[0]));
-      v.z = __ldg(rowp + clamp_to(gx0 + 2, dimx, ib.lo[0], ib.n[0]));
-      v.w = __ldg(rowp + clamp_to(gx0 + 3, dimx, ib.lo[0], ib.n[0]));
+      v.x = __ldca(rowp + clamp_to(gx0, dimx, ib.lo[0], ib.n[0]));
+      v.y = __ldca(rowp + clamp_to(gx0 + 1, dimx, ib.lo[0], ib.n[0]));
+      v.z = __ldca(rowp + clamp_to(gx0 + 2, dimx, ib.lo[0], ib.n[0]));
+      v.w = __ldca(rowp + clamp_to(gx0 + 3, dimx, ib.lo[0], ib.n[0]));
     }
     *reinterpret_cast<float4*>(&sin_[comp][row][4 * cq]) = v;
   }
@@ -204,7 +204,7 @@ __device__ __forceinline__ void rho_stream_body(const float* __restrict__ in, Bo
 
   float win[WN];
 #pragma unroll
-  for (int j = 0; j < 2 * RR; ++j) win[j] = __ldg(src(j));
+  for (int j = 0; j < 2 * RR; ++j) win[j] = __ldca(src(j));
   // blocks 0 and 1: steps 2R + t, t < 2 kT, into ring slot t
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
@@ -376,7 +376,7 @@ __global__ void __launch_bounds__(kZ2Threads, RR >= 32 ? 2 : 3)
   };
   float2 win[WN];
 #pragma unroll
-  for (int j = 0; j < 2 * RR; ++j) win[j] = __ldg(reinterpret_cast<const float2*>(src(j)));
+  for (int j = 0; j < 2 * RR; ++j) win[j] = __ldca(reinterpret_cast<const float2*>(src(j)));
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
 #pragma unroll

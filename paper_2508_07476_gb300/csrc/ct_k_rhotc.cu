@@ -575,8 +575,8 @@ __global__ void __launch_bounds__(TcRoles<XAXIS, PROD>::THREADS, 1)
             if (two)
               cp_async4(smem_u32(sb + j * kTcLines + m), reinterpret_cast<const float*>(gbase + IU.gb + q));
           } else {  // FP16: below the 4-byte copy size, loaded and stored here
-            sa[j * kTcLines + m] = gbase[IU.ga + q];
-            if (two) sb[j * kTcLines + m] = gbase[IU.gb + q];
+            sa[j * kTcLines + m] = __ldca(gbase + IU.ga + q);
+            if (two) sb[j * kTcLines + m] = __ldca(gbase + IU.gb + q);
           }
         }
       }
