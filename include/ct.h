@@ -381,9 +381,11 @@ ct_status ct_track(const ct_track_params* params, const int64_t vol_dims[3], con
  * current device, on a seeded synthetic annulus of that size (with the
  * annulus mask when `masked`), one padded-box call per candidate over the
  * whole volume, or over a chunk of size `chunk` (nullable; 0 = whole extent)
- * at the volume's centre with its halo, as ct_run_chunks processes chunks: the rho passes as FP32 stencils (8 or 16 outputs per y / z thread
- * block) or on the tensor cores (products formed in the gradient kernel or in
- * the first pass; work units of at most 512, 256 or 128 outputs), then, when
+ * at the volume's centre with its halo, as ct_run_chunks processes chunks: the
+ * rho passes as FP32 stencils (where the z pass runs over rows of odd length, with
+ * blocks of 8 and of 16 outputs per thread) or on the tensor cores (products formed in
+ * the gradient kernel or in the first pass; work units of at most 512, 256 or
+ * 128 outputs), then, when
  * masked, the eigen stage over compacted voxels or a thread per voxel.  Best
  * of 3 runs after a warm-up, CUDA events.  *out gets the best choice, its
  * time and that of the built-in choices.  With cache_file (nullable) the
@@ -403,7 +405,7 @@ typedef struct ct_tune_result {
   int32_t rho_path;     /* 0 FP32 stencils; 1 tensor cores, products in the gradient kernel;
                            2 tensor cores, products formed in the first pass */
   int32_t seg_cap;      /* tensor-core outputs per work unit at most (0: not tuned) */
-  int32_t stream_block; /* stencil outputs per y / z thread block (0: not tuned) */
+  int32_t stream_block; /* outputs per thread and block of the z stencil over odd rows (0: not tuned) */
   int32_t eig_compact;  /* 1 compacted, 0 a thread per voxel, -1 not tuned (unmasked) */
   double ms;            /* best time of one run */
   double default_ms;    /* time with the built-in choices */

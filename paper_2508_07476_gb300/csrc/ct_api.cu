@@ -199,7 +199,7 @@ struct ct_plan_s {
   uint64_t ready_s = 0, ready_r = 0;  // radii whose kernels' attributes are set (ensure_kernels)
   ct_stats stats;
   std::mutex mu;
-  int stream_block = 16;  // outputs per thread block of k_rho_stream: y, or z over odd rows (tuning choice)
+  int stream_block = 16;  // k_rho_stream's outputs per thread and block: y, or z over odd rows (tuning choice)
   int tc_rho = 7;           // rho passes on the tensor cores: bit a for axis a (tuning choice)
   int tc_min_r = 24;        // ... for rho radii of at least this (tuning choice)
   int64_t tc_min_vox = int64_t(1) << 24;  // ... on volumes of at least this many voxels (tuning choice)
@@ -216,7 +216,7 @@ struct ct_plan_s {
     int rho_path;      // 0: FP32 stencils; 1: tensor cores, products in the gradient kernel;
                        // 2: tensor cores, products formed in the first pass
     int seg_cap;       // tensor-core outputs per work unit at most (0: the default)
-    int stream_block;  // k_rho_stream's outputs per thread block (0: the default)
+    int stream_block;  // k_rho_stream's outputs per thread and block (0: the default)
     int eig_compact;   // masked eigen stage over compacted voxels (-1: the default)
     double ms;
   };
@@ -2029,7 +2029,12 @@ ct_status ct_autotune(const ct_params* params, const int64_t vol_dims[3], const 
   if (xc >= 4)  // the tensor-core passes' 16-byte copies want x extents that are multiples of 4
     for (int path : {2, 1})
       for (int seg : {512, 256, 128}) cands.push_back(entry(path, seg, 0, -1));
-  for (int sb : {16, 8}) cands.push_back(entry(0, 0, sb, -1));
+  // k_rho_stream runs the stencil chain's z pass over rows of odd length alone: elsewhere its
+  // block size names no kernel of the chain, and one candidate stands for the stencils
+  if (chain_boxes(sc, dims, ib, ob, true).S.n[0] % 2 != 0)
+    for (int sb : {16, 8}) cands.push_back(entry(0, 0, sb, -1));
+  else
+    cands.push_back(entry(0, 0, 0, -1));
   ct_plan_s::TuneEntry best = cands[0];
   best.ms = 1e30;
   for (auto& c : cands) {

@@ -1,6 +1,6 @@
-"""Scratch of a plan across its calls, on the host alone: the library's objects
-linked with a double of the CUDA runtime (cudart_double.cpp), which counts what
-the plan allocates, frees, captures and launches."""
+"""Scratch of a plan across its calls and the tuner's candidates, on the host alone: the library's
+objects linked with a double of the CUDA runtime (cudart_double.cpp), which counts
+what the plan allocates, frees, captures and launches."""
 import ctypes
 import os
 import shutil
@@ -147,3 +147,16 @@ def test_a_first_call_allocates_its_scratch_once(plan):
     plan.box(WIDE)
     after = plan.counts()
     assert after[MALLOCS] - before[MALLOCS] == 5 and after[FREES] == before[FREES]
+
+
+@pytest.mark.parametrize("nx,blocks", [(62, 1), (63, 2), (64, 1), (65, 1), (161, 1)])
+def test_the_tuner_times_a_block_size_only_where_a_kernel_takes_it(lib, nx, blocks):
+    """The z pass over rows of odd length (narrow boxes: wider rows are padded) alone has two block
+    sizes to choose from; elsewhere the stencils are one candidate, its block size not tuned."""
+    params = _lib.make_params(1.0, 3.0, (0.0, 0.0, 0.0), (0.0, 0.0, 1.0))
+    r = _lib.ct_tune_result()
+    assert lib.ct_autotune(ctypes.byref(params), _lib._i64x3((nx, 40, 30)), None, 0, None, ctypes.byref(r)) == 0
+    tensor_core = 6 if nx % 4 == 0 else 0
+    assert r.candidates == 1 + tensor_core + blocks
+    if not tensor_core:
+        assert r.rho_path == 0 and (r.stream_block > 0) == (blocks == 2)
