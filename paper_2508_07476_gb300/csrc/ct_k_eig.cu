@@ -92,11 +92,13 @@ __device__ __forceinline__ void push_fallback(const Fallback& fb, int64_t i) {
 #ifndef CT_EIG_MINB
 #define CT_EIG_MINB 8
 #endif
+// Rows from which on the re-solve's CTAs may start while the stage still runs (after_previous).
+constexpr int kEigStartNextMinX = 96;
 template <int VT, int AT, int FT>
 __global__ void __launch_bounds__(256, CT_EIG_MINB)
     k_eig_angles(const float* __restrict__ S, Box sb, Box ob, const uint8_t* __restrict__ mask, Box mb, Frame F,
                  float fill, EigOut o, bool mixed, Fallback fb) {
-  after_previous();
+  after_previous(ob.n[0] >= kEigStartNextMinX);
   const int x = ob.lo[0] + blockIdx.x * blockDim.x + threadIdx.x;
   if (x >= ob.lo[0] + ob.n[0]) return;
   const int row = blockIdx.z * gridDim.y + blockIdx.y;  // y + ny * z within ob
@@ -148,7 +150,7 @@ __global__ void __launch_bounds__(256, CT_EIG_MINB)
     k_eig_angles32(const float* __restrict__ S, Box sb, Box ob, const uint8_t* __restrict__ mask, Box mb, Frame F,
                    float fill, EigOut o, bool mixed, Fallback fb) {
   (void)mixed;
-  after_previous();
+  after_previous(ob.n[0] >= kEigStartNextMinX);
   eig32_body<VT, AT, FT, PLAIN>(S, sb, ob, mask, mb, F, fill, o, fb, HwBlock{});
 }
 
@@ -164,7 +166,7 @@ constexpr int kEigRowSpan = 8 * kEigRowThreads;
 template <int VT, int AT, int FT, bool PLAIN>
 __global__ void __launch_bounds__(kEigRowThreads, 24)
     k_eig_angles_rows(const float* __restrict__ S, Box sb, Box ob, Frame F, float fill, EigOut o, Fallback fb) {
-  after_previous();
+  after_previous(ob.n[0] >= kEigStartNextMinX);
   const int y = ob.lo[1] + blockIdx.y, z = ob.lo[2] + blockIdx.z;
   const int x0 = ob.lo[0] + blockIdx.x * kEigRowSpan;
   const int xend = min(ob.lo[0] + ob.n[0], x0 + kEigRowSpan);
@@ -290,7 +292,7 @@ __global__ void __launch_bounds__(kEigThreads, CT_EIG_MINB * 256 / kEigThreads)
     k_eig_angles_compact(const float* __restrict__ S, Box sb, Box ob, const uint8_t* __restrict__ mask, Box mb,
                          Frame F, float fill, EigOut o, bool mixed, Fallback fb) {
   (void)mixed;
-  after_previous();
+  after_previous(ob.n[0] >= kEigStartNextMinX);
   eig_compact_body<VT, AT, FT, PLAIN>(S, sb, ob, mask, mb, F, fill, o, fb, HwBlock{});
 }
 

@@ -18,9 +18,9 @@ cudaError_t prepare_grad_split_kernels(int rk);
 
 // Where a kernel of the chain goes: the stream, and whether its CTAs may be
 // scheduled while the stream's previous kernel drains (`early`; every kernel
-// launched through launch_after begins with after_previous(), which waits for that
-// kernel).  That hides the launch latency of a chain of short kernels (64^3: 50 ->
-// 40 us; 173 x 141 x 118: 207 -> 195; a 256^3 chunk: 1118 -> 1099), but an SM that
+// launched through launch_after waits for that kernel first: after_previous()).
+// That hides the launch latency of a chain of short kernels (64^3: 50 -> 40 us;
+// 173 x 141 x 118: 207 -> 195; a 256^3 chunk: 1118 -> 1099), but an SM that
 // never drains keeps its split of L1 and shared memory: the eigen stage after a
 // tensor-core pass then runs with little L1 (512^3: 4837 -> 4949 us; a 384^3 chunk,
 // 57M voxels: even), and beside other streams the waiting CTAs hold room those could

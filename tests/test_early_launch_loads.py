@@ -15,7 +15,7 @@ STEADY = r"(reinterpret_cast<const (uint32_t|float4)\*>\()?(mask|evals|evec)\b"
 def test_chain_inputs_are_read_by_plain_loads(name):
     with open(os.path.join(build.CSRC, name)) as f:
         code = re.sub(r"//[^\n]*", "", f.read())
-    assert "after_previous();" in code
+    assert "after_previous(" in code
     assert [m for m in re.findall(r"__ldg\(([^;]*);", code) if not re.match(STEADY, m)] == []
     if name == "ct_k_rhotc.cu":  # element copies of the gradient
         assert not re.search(r"= gbase\[", code)
