@@ -976,10 +976,24 @@ std::vector<Box> chunk_grid(const int dims[3], const int64_t chunk[3]) {
   return out;
 }
 
-// 3D copy of box `b` between an array covering `arr` (x-fastest, element size
-// esz) and a dense array covering exactly `b`.
+// Copy of box `b` between an array covering `arr` (x-fastest, element size esz)
+// and a dense array covering exactly `b`: one range where the box holds whole
+// planes, a row per plane where it holds whole rows of part of them, and a 3-D
+// copy else.  The 3-D copy runs at a small fraction of the link's rate unless its
+// rows are of certain lengths, whatever the box: 300 x 256 x 64 in slabs of 8
+// planes, F32 outputs, 5290 us so and 2140 as ranges (256 x 256 planes 3200 either way).
 cudaError_t copy_box(const void* src, void* dst, const Box& arr, const Box& b, size_t esz, bool to_device,
                      cudaStream_t st) {
+  const cudaMemcpyKind kind = to_device ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToHost;
+  if (b.n[0] == arr.n[0]) {
+    const size_t row = esz * arr.n[0], run = row * b.n[1], plane = row * arr.n[1];
+    const size_t off = row * (b.lo[1] - arr.lo[1]) + plane * (b.lo[2] - arr.lo[2]);
+    const char* from = (const char*)src + (to_device ? off : 0);
+    char* to = (char*)dst + (to_device ? 0 : off);
+    if (run == plane || b.n[2] == 1) return cudaMemcpyAsync(to, from, run * b.n[2], kind, st);
+    if (plane <= 0x7fffffff)  // (the largest pitch of a 2-D copy)
+      return cudaMemcpy2DAsync(to, to_device ? run : plane, from, to_device ? plane : run, run, b.n[2], kind, st);
+  }
   cudaMemcpy3DParms p;
   std::memset(&p, 0, sizeof p);
   cudaPitchedPtr whole = make_cudaPitchedPtr(const_cast<void*>(to_device ? src : dst), esz * arr.n[0], arr.n[0],
@@ -990,13 +1004,12 @@ cudaError_t copy_box(const void* src, void* dst, const Box& arr, const Box& b, s
     p.srcPtr = whole;
     p.srcPos = pos;
     p.dstPtr = dense;
-    p.kind = cudaMemcpyHostToDevice;
   } else {
     p.srcPtr = dense;
     p.dstPtr = whole;
     p.dstPos = pos;
-    p.kind = cudaMemcpyDeviceToHost;
   }
+  p.kind = kind;
   p.extent = make_cudaExtent(esz * b.n[0], b.n[1], b.n[2]);
   return cudaMemcpy3DAsync(&p, st);
 }

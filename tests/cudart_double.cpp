@@ -18,7 +18,7 @@ std::map<char*, size_t> live;  // device blocks
 size_t limit = SIZE_MAX;       // a larger device block is refused
 bool own_capture = false;      // between cudaStreamBeginCapture and EndCapture
 bool user_capture = false;     // the caller's stream captures
-int64_t mallocs = 0, frees = 0, instantiated = 0, graph_launches = 0, stale_launches = 0;
+int64_t mallocs = 0, frees = 0, instantiated = 0, graph_launches = 0, stale_launches = 0, strided = 0;
 
 struct Graph {
   std::set<char*> blocks;  // the blocks that were live when it was captured
@@ -39,9 +39,9 @@ extern "C" {
 void double_limit(uint64_t bytes) { limit = bytes; }
 void double_user_capture(int on) { user_capture = on != 0; }
 // 0 allocations, 1 frees, 2 graphs instantiated, 3 graph launches, 4 launches of a
-// graph one of whose blocks was freed after its capture
+// graph one of whose blocks was freed after its capture, 5 copies row by row (3-D)
 int64_t double_count(int k) {
-  const int64_t v[] = {mallocs, frees, instantiated, graph_launches, stale_launches};
+  const int64_t v[] = {mallocs, frees, instantiated, graph_launches, stale_launches, strided};
   return v[k];
 }
 
@@ -63,15 +63,21 @@ cudaError_t cudaFree(void* p) {
   return cudaSuccess;
 }
 cudaError_t cudaFreeHost(void*) { return cudaSuccess; }
+// The words that the library itself reads back (counters) are zero; arrays are not written.
 cudaError_t cudaMemcpy(void* d, const void*, size_t n, cudaMemcpyKind kind) {
-  if (kind == cudaMemcpyDeviceToHost) std::memset(d, 0, n);
+  if (kind == cudaMemcpyDeviceToHost && n <= 8) std::memset(d, 0, n);
   return cudaSuccess;
 }
-cudaError_t cudaMemcpyAsync(void* d, const void*, size_t n, cudaMemcpyKind kind, cudaStream_t) {
-  if (kind == cudaMemcpyDeviceToHost) std::memset(d, 0, n);
+cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind kind, cudaStream_t) {
+  return cudaMemcpy(d, s, n, kind);
+}
+cudaError_t cudaMemcpy2DAsync(void*, size_t dp, const void*, size_t sp, size_t w, size_t, cudaMemcpyKind, cudaStream_t) {
+  return w <= dp && w <= sp && dp <= 0x7fffffff && sp <= 0x7fffffff ? cudaSuccess : cudaErrorInvalidPitchValue;
+}
+cudaError_t cudaMemcpy3DAsync(const cudaMemcpy3DParms*, cudaStream_t) {
+  ++strided;
   return cudaSuccess;
 }
-cudaError_t cudaMemcpy3DAsync(const cudaMemcpy3DParms*, cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaMemset(void*, int, size_t) { return cudaSuccess; }
 cudaError_t cudaMemsetAsync(void*, int, size_t, cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaGetSymbolAddress(void** p, const void*) { return token(p); }

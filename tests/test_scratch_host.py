@@ -1,6 +1,7 @@
-"""Scratch of a plan across its calls and the tuner's candidates, on the host alone: the library's
-objects linked with a double of the CUDA runtime (cudart_double.cpp), which counts
-what the plan allocates, frees, captures and launches."""
+"""Scratch of a plan across its calls, the tuner's candidates and the copies of host items, on the
+host alone: the library's objects linked with a double of the CUDA runtime
+(cudart_double.cpp), which counts what the plan allocates, frees, captures, launches and
+copies."""
 import ctypes
 import os
 import shutil
@@ -11,7 +12,7 @@ import pytest
 from paper_2508_07476_gb300 import _lib, build
 
 HERE = os.path.dirname(os.path.abspath(__file__))
-MALLOCS, FREES, INSTANTIATED, LAUNCHED, STALE = range(5)
+MALLOCS, FREES, INSTANTIATED, LAUNCHED, STALE, STRIDED = range(6)
 ADDRESS = 1 << 20  # a device address: the double's kernels read and write nothing
 
 
@@ -35,9 +36,9 @@ def lib(tmp_path_factory):
 class Plan:
     """A plan on the double, and what its calls cost."""
 
-    def __init__(self, lib, dims, rho=3.0):
+    def __init__(self, lib, dims, rho=3.0, chunk=(0, 0, 0)):
         self.lib, self.dims, self.p = lib, dims, ctypes.c_void_p()
-        params = _lib.make_params(1.0, rho, (300.0, 260.0, 10.0), (0.1, 0.1, 1.0), _lib.CT_PREC_MIXED)
+        params = _lib.make_params(1.0, rho, (300.0, 260.0, 10.0), (0.1, 0.1, 1.0), _lib.CT_PREC_MIXED, chunk=chunk)
         self.ok(lib.ct_plan_create(ctypes.byref(params), _lib._i64x3(dims), ctypes.byref(self.p)))
 
     def ok(self, status):
@@ -56,7 +57,7 @@ class Plan:
         self.ok(self.lib.ct_eig_smallest(self.p, ADDRESS, n, ADDRESS, ADDRESS, None))
 
     def counts(self):
-        return [self.lib.double_count(k) for k in range(5)]
+        return [self.lib.double_count(k) for k in range(6)]
 
 
 @pytest.fixture
@@ -160,3 +161,22 @@ def test_the_tuner_times_a_block_size_only_where_a_kernel_takes_it(lib, nx, bloc
     assert r.candidates == 1 + tensor_core + blocks
     if not tensor_core:
         assert r.rho_path == 0 and (r.stream_block > 0) == (blocks == 2)
+
+
+@pytest.mark.parametrize("chunk,slab_bytes,strided", [
+    ((0, 0, 0), None, False), ((0, 0, 8), None, False), ((0, 33, 8), None, False), ((64, 33, 8), None, False),
+    ((64, 33, 8), "1000000", True)])
+@pytest.mark.parametrize("masked", [False, True])
+def test_host_copies_of_whole_rows_are_no_strided_copies(lib, monkeypatch, chunk, slab_bytes, strided, masked):
+    """Slabs of whole rows are copied as ranges, or a range per plane; only runs cut along x (here by
+    the slab's bytes) are copied row by row."""
+    if slab_bytes:
+        monkeypatch.setenv("CT_TUNE_SLAB_BYTES", slab_bytes)
+    plan = Plan(lib, (161, 90, 40), chunk=chunk)
+    try:
+        before = plan.counts()
+        item = _lib.make_item(ADDRESS, plan.dims, ADDRESS if masked else None, ADDRESS, ADDRESS, ADDRESS, ADDRESS)
+        plan.ok(lib.ct_run_chunks(plan.p, (_lib.ct_item * 1)(item), 1, 1, None))
+        assert (plan.counts()[STRIDED] > before[STRIDED]) == strided
+    finally:
+        lib.ct_plan_destroy(plan.p)
