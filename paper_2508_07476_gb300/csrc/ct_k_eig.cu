@@ -163,6 +163,17 @@ __global__ void __launch_bounds__(256, CT_EIG_MINB)
 // per SM instead of 24, at 32 / 42 registers: 6.24).
 constexpr int kEigRowThreads = 64;
 constexpr int kEigRowSpan = 8 * kEigRowThreads;
+// Whether rows of n voxels without a mask take k_eig_angles_rows.  It walks a row in steps of
+// two warps: 1, 3 or 5 warps of voxels leave half a CTA idle in one of few steps, and a short
+// second span a CTA with little to do; those take a thread per voxel.  12000 / n x n x 300
+// voxels, F16 outputs, rows against threads: 24 columns 117 and 84 us, 72 74 and 63, 96 58 and
+// 51, 140 57 and 56, 530 54 and 50; but 64 49 and 54, 128 45 and 49, 173 49 and 55,
+// 256 45 and 49, 384 45 and 49, 1000 47 and 51.
+static bool eig_rows(int n) {
+  const int warps = (n + 31) / 32, last = n % kEigRowSpan;
+  return warps != 1 && warps != 3 && warps != 5 && !(n > kEigRowSpan && last > 0 && last <= 128);
+}
+
 template <int VT, int AT, int FT, bool PLAIN>
 __global__ void __launch_bounds__(kEigRowThreads, 24)
     k_eig_angles_rows(const float* __restrict__ S, Box sb, Box ob, Frame F, float fill, EigOut o, Fallback fb) {
@@ -414,7 +425,7 @@ cudaError_t launch_eig_angles(const float* S, const Box& sb, const Box& ob, cons
                             fb);
       }
     }
-    if (mask == nullptr && plain) {  // k_eig_angles_rows has both forms' times
+    if (mask == nullptr && plain && eig_rows(ob.n[0])) {
       const dim3 gr((ob.n[0] + kEigRowSpan - 1) / kEigRowSpan, ob.n[1], ob.n[2]);
       if (o.vec_t == CT_OUT_F32 && o.ang_t == CT_OUT_F32 && o.fa_t == CT_OUT_F32)
         return launch_after(k_eig_angles_rows<0, 0, 0, true>, gr, kEigRowThreads, 0, st, S, sb, ob, F, fill, o, fb);
