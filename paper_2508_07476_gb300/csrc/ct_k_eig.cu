@@ -632,8 +632,8 @@ __device__ __forceinline__ void store_angles(void* base, IT i, int type, const f
 // Every array of the stage is dense over the box, so a thread takes V
 // consecutive voxels of the flat index: one division of it for the first
 // voxel's position, the others by stepping.  V = 4 (16-byte loads and stores)
-// where every plane keeps that alignment; nothing is read for a group that
-// lies outside the mask.  256^3, F16 outputs, a wall's mask: 142 us with
+// where every plane keeps that alignment and the threads still fill the GPU
+// (kAnglesVecMin); nothing is read for a group that lies outside the mask.  256^3, F16 outputs, a wall's mask: 142 us with
 // 64-bit divisions per voxel, encodings read at run time and every voxel's
 // vector loaded, 94 us now, bound by the instructions of the inside voxels'
 // angles (its 403 MB take 59 us at the copy rate).
@@ -731,6 +731,11 @@ static cudaError_t angles_t(const float* evec, const float* evals, const Box& ob
   return cudaGetLastError();
 }
 
+// Four voxels per thread from so many voxels on.  Below, a voxel per thread takes less, as
+// more threads share its latency: 32^3 F32 2.0 against 3.1 us (2.5 with 64-bit indices), 48^3
+// 2.5 and 3.2, 60^3 3.7 and 3.9; 64^3 4.0 and 3.9, 80^3 6.3 and 5.4.
+constexpr int64_t kAnglesVecMin = (int64_t)1 << 18;
+
 template <int VT, int AT, int FT>
 static cudaError_t angles_e(const float* evec, const float* evals, const Box& ob, const uint8_t* mask,
                             const Frame& F, float fill, const EigOut& o, bool vec4, bool plain, cudaStream_t st) {
@@ -749,10 +754,11 @@ cudaError_t launch_angles_only(const float* evec, const float* evals, const Box&
   if (3 * n >= ((int64_t)1 << 31) - ((int64_t)1 << 24))
     return angles_t<-1, -1, -1, false, 1, int64_t>(evec, evals, ob, mask, F, fill, o, st);
   // four voxels per thread where all planes of all arrays start on the boundary
-  // of four elements (a plane of n elements keeps it for the next when n does)
+  // of four elements (a plane of n elements keeps it for the next when n does) and
+  // there are enough of them
   auto at = [](const void* p, uintptr_t b) { return reinterpret_cast<uintptr_t>(p) % b == 0; };
   auto size = [](int t) { return (uintptr_t)(t == CT_OUT_F32 ? 4 : t == CT_OUT_F16 ? 2 : 1); };
-  const bool vec4 = n % 4 == 0 && at(evec, 16) && at(evals, 16) && at(mask, 4) && at(o.vec, 4 * size(o.vec_t)) &&
+  const bool vec4 = n >= kAnglesVecMin && n % 4 == 0 && at(evec, 16) && at(evals, 16) && at(mask, 4) && at(o.vec, 4 * size(o.vec_t)) &&
                     at(o.ha, 4 * size(o.ang_t)) && at(o.ia, 4 * size(o.ang_t)) && at(o.fa, 4 * size(o.fa_t));
   const bool plain = F.sp[0] == 1.f && F.sp[1] == 1.f && F.sp[2] == 1.f && F.centres == nullptr;
   if (o.vec_t == CT_OUT_F32 && o.ang_t == CT_OUT_F32 && o.fa_t == CT_OUT_F32)
