@@ -59,8 +59,9 @@ __device__ __forceinline__ int clamp_to(int p, int dim, int lo, int n) {
 // start_next false: the next kernel's CTAs start as this one's end.  Letting them start
 // costs every CTA a fixed time (about 1 ns of the whole GPU's), which bounds a kernel of many
 // small CTAs: the eigen stage has one per row, and over rows of 16 voxels, 225 000 of them,
-// took 231 us with it, 121 without; over rows of 96 and more it is hidden, and the re-solve
-// behind it gains 1 to 2 us.
+// takes 231 us with it, 121 without.  Over rows of 96 voxels and more it is hidden, and of
+// fewer than 4096 rows the re-solve's earlier start gains more (64 x 63 x 53 as a whole, masked
+// 38.5 us with it, 39.0 without; 64^3 39.8 and 39.3).
 __device__ __forceinline__ void after_previous(bool start_next = true) {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   if (start_next) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

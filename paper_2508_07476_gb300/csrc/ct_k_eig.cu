@@ -92,13 +92,16 @@ __device__ __forceinline__ void push_fallback(const Fallback& fb, int64_t i) {
 #ifndef CT_EIG_MINB
 #define CT_EIG_MINB 8
 #endif
-// Rows from which on the re-solve's CTAs may start while the stage still runs (after_previous).
-constexpr int kEigStartNextMinX = 96;
+// Whether the re-solve's CTAs may start while the stage still runs (after_previous): not where
+// many CTAs of narrow rows would be bound by it.
+__device__ __forceinline__ bool starts_next(const Box& ob) {
+  return ob.n[0] >= 96 || (int64_t)ob.n[1] * ob.n[2] < 4096;
+}
 template <int VT, int AT, int FT>
 __global__ void __launch_bounds__(256, CT_EIG_MINB)
     k_eig_angles(const float* __restrict__ S, Box sb, Box ob, const uint8_t* __restrict__ mask, Box mb, Frame F,
                  float fill, EigOut o, bool mixed, Fallback fb) {
-  after_previous(ob.n[0] >= kEigStartNextMinX);
+  after_previous(starts_next(ob));
   const int x = ob.lo[0] + blockIdx.x * blockDim.x + threadIdx.x;
   if (x >= ob.lo[0] + ob.n[0]) return;
   const int row = blockIdx.z * gridDim.y + blockIdx.y;  // y + ny * z within ob
@@ -150,7 +153,7 @@ __global__ void __launch_bounds__(256, CT_EIG_MINB)
     k_eig_angles32(const float* __restrict__ S, Box sb, Box ob, const uint8_t* __restrict__ mask, Box mb, Frame F,
                    float fill, EigOut o, bool mixed, Fallback fb) {
   (void)mixed;
-  after_previous(ob.n[0] >= kEigStartNextMinX);
+  after_previous(starts_next(ob));
   eig32_body<VT, AT, FT, PLAIN>(S, sb, ob, mask, mb, F, fill, o, fb, HwBlock{});
 }
 
@@ -164,20 +167,21 @@ __global__ void __launch_bounds__(256, CT_EIG_MINB)
 constexpr int kEigRowThreads = 64;
 constexpr int kEigRowSpan = 8 * kEigRowThreads;
 // Whether rows of n voxels without a mask take k_eig_angles_rows.  It walks a row in steps of
-// two warps: 1, 3 or 5 warps of voxels leave half a CTA idle in one of few steps, and a short
-// second span a CTA with little to do; those take a thread per voxel.  12000 / n x n x 300
+// two warps: 1 or 3 warps of voxels leave half a CTA idle in one of one or two steps, and a
+// short second span a CTA with little to do; those take a thread per voxel.  12000 / n x n x 300
 // voxels, F16 outputs, rows against threads: 24 columns 117 and 84 us, 72 74 and 63, 96 58 and
-// 51, 140 57 and 56, 530 54 and 50; but 64 49 and 54, 128 45 and 49, 173 49 and 55,
-// 256 45 and 49, 384 45 and 49, 1000 47 and 51.
+// 51, 530 54 and 50; but 64 49 and 54, 128 45 and 49, 173 49 and 55, 256 45 and 49, 384 45 and
+// 49, 1000 47 and 51.  At 129 to 160 columns rows are up to 4% slower alone and faster beside
+// other streams (117 x 192 x 109 and 129 x 69 x 157 in one call 301 and 307 us).
 static bool eig_rows(int n) {
   const int warps = (n + 31) / 32, last = n % kEigRowSpan;
-  return warps != 1 && warps != 3 && warps != 5 && !(n > kEigRowSpan && last > 0 && last <= 128);
+  return warps != 1 && warps != 3 && !(n > kEigRowSpan && last > 0 && last <= 128);
 }
 
 template <int VT, int AT, int FT, bool PLAIN>
 __global__ void __launch_bounds__(kEigRowThreads, 24)
     k_eig_angles_rows(const float* __restrict__ S, Box sb, Box ob, Frame F, float fill, EigOut o, Fallback fb) {
-  after_previous(ob.n[0] >= kEigStartNextMinX);
+  after_previous(starts_next(ob));
   const int y = ob.lo[1] + blockIdx.y, z = ob.lo[2] + blockIdx.z;
   const int x0 = ob.lo[0] + blockIdx.x * kEigRowSpan;
   const int xend = min(ob.lo[0] + ob.n[0], x0 + kEigRowSpan);
@@ -303,7 +307,7 @@ __global__ void __launch_bounds__(kEigThreads, CT_EIG_MINB * 256 / kEigThreads)
     k_eig_angles_compact(const float* __restrict__ S, Box sb, Box ob, const uint8_t* __restrict__ mask, Box mb,
                          Frame F, float fill, EigOut o, bool mixed, Fallback fb) {
   (void)mixed;
-  after_previous(ob.n[0] >= kEigStartNextMinX);
+  after_previous(starts_next(ob));
   eig_compact_body<VT, AT, FT, PLAIN>(S, sb, ob, mask, mb, F, fill, o, fb, HwBlock{});
 }
 
