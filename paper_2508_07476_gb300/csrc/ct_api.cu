@@ -449,14 +449,15 @@ const ct_plan_s::TuneEntry* tuned(const ct_plan P, const Scale& sc, const int di
 // a function of the plan, the volume's extent and the scale, never of the box,
 // so that every chunk and sub-box of a volume takes the same arithmetic as the
 // whole and their results agree bit for bit.  Those passes are bound by HBM at
-// 48 B per voxel with 16-byte copies (x extents that are multiples of 4) and
-// several times slower otherwise; the FP32 stencils cost 6 (2R+1) FMAs per
-// voxel and pass, so below R ~ 17 they are the faster, and on small volumes
-// the persistent passes' start-up outweighs them (one step: 200^3 0.87 ms on
-// the tensor cores against 0.72 on the stencils; 256^3 0.98 against 1.12;
-// 384^3 2.70 against 3.34; 400^3 3.91 against 4.23; 200 uneven crops, all on
-// the tensor cores where the extent allows, 167 ms against 164).  tc_any_box
-// drops the extent and size conditions (tests drive every copy path with it).
+// 48 B per voxel where their copies are 16 bytes wide (the x pass wants x extents that
+// are multiples of 4, the passes over z and y groups of 32 whole columns) and slower
+// otherwise; the FP32 stencils cost 6 (2R+1) FMAs per voxel and pass, so below R ~ 17
+// they are the faster, and on small volumes of such extents too.  One mixed step, sigma
+// 2, rho 6, tensor cores and stencils: 128^3 0.15 and 0.17 ms, 200^3 0.70 and 0.61, 232^3
+// 0.86 and 0.80, 256^3 0.73 and 0.95, 384^3 2.14 and 2.91, 400^3 3.82 and 3.83; 200 uneven
+// crops, all on the tensor cores where R and the extent allow, 133.3 ms, on stencils
+// alone 129.4.  tc_any_box drops the extent and size conditions (tests drive every
+// copy path with it).
 bool use_tc(const ct_plan P, const Scale& sc, const int dims[3], int axis) {
   if (const auto* t = tuned(P, sc, dims)) return t->rho_path > 0;
   const int64_t vox = (int64_t)dims[0] * dims[1] * dims[2];
@@ -1098,9 +1099,9 @@ uint64_t fnv1a(uint64_t h, const void* data, size_t n) {
 // rho x/y, rho z) that runs in order on one of the plan's streams, chains side
 // by side; the eigen stage of the whole wave follows them.  A wave holds the items whose scratch (the two tensor
 // buffers and the re-solve list) fits the plan's batch_bytes; waves reuse the
-// arena in stream order.  Every item's blocks, launch shape and arithmetic are
-// those of its single launch, so a batch reproduces each item alone bit for
-// bit.  The launch records (tables in device memory, uploaded before any
+// arena in stream order.  Every output's arithmetic is that of the item's single
+// launch (their CTA shapes and scratch rows may differ), so a batch reproduces
+// each item alone bit for bit.  The launch records (tables in device memory, uploaded before any
 // capture) are built here; run_persistent_waves enqueues them.
 struct MultiRec {
   int kind;          // 0 grad_xy, 1 grad_z, 2 rho_xy, 3 rho_z, 4 eigen (compact), 5 eigen (per voxel)
@@ -1278,7 +1279,7 @@ ct_status build_persistent_waves(ct_plan P, const ct_item* items, const std::vec
       }
       {
         RxyItem x{A, G, c.dims[0], c.dims[1], B, Bxy, 0};
-        const int xt = rho_xy_width(Bxy.n[0]);  // the single launch's CTA width (items of each width in one launch)
+        const int xt = rho_xy_width(Bxy.n[0]);  // items of each CTA width in one launch
         g_rxy.push_back(rho_xy_item(c.sc.rkr, xt, x));
         rxy.push_back(x);
         MultiRec r = base;
@@ -1296,7 +1297,7 @@ ct_status build_persistent_waves(ct_plan P, const ct_item* items, const std::vec
         r.kind = 3;
         r.rk = c.sc.rkr;
         r.block_t = t && t->stream_block ? t->stream_block : P->stream_block;
-        r.block = rho_stream_block(ob, 2);  // the single launch's CTA shape (items of each shape in one launch)
+        r.block = rho_stream_block(ob, 2);  // items of each CTA shape in one launch
         r.t0 = c.sc.tr[2];
         g_rz.push_back(rho_z_item(c.sc.rkr, r.block_t, r.block, x));
         rz.push_back(x);
@@ -1687,16 +1688,16 @@ ct_status run_device_batch(ct_plan P, const ct_item* items, int n, cudaStream_t 
 // two streams, so the copies of one overlap the kernels of the other; stream
 // order protects each slot's outputs.  The copies to the device go through a
 // stream of their own, a slab's as soon as the kernels that read its buffer
-// are done: behind that slab's copies to the host, in the slot's stream, they kept the
+// are done: behind that slab's copies to the host, in the slot's stream, they keep the
 // next kernels waiting and the link to the host idle (512 x 512 x 256, F16 outputs,
-// slabs of 64 planes: 6.40 -> 5.90 ms; its outputs alone take 4.2 ms of the link).
+// slabs of 64 planes: 6.40 ms so, 5.90 in their own; its outputs take 4.2 ms of the link).
 // Every chunk's arithmetic is that of a chunk on its own, so the results equal the
 // whole volume's bit for bit.
 constexpr int kUpStream = 2;  // the stream of the host-to-device copies
 // A slab of at least so many voxels also waits for the kernels of the one before: side
 // by side the two finish late together, one after the other the first one's outputs
-// leave while the second is computed (the volume above 5.90 -> 5.70 ms; 256 x 256 x 128 in
-// 128 x 128 x 64 chunks 1.65 -> 1.46).  Smaller slabs do not fill the GPU alone
+// leave while the second is computed (the volume above 5.90 and 5.70 ms; 256 x 256 x 128 in
+// 128 x 128 x 64 chunks 1.65 and 1.46).  Smaller slabs do not fill the GPU alone
 // (128 x 128 x 32: 0.537 side by side, 0.545 ms in turn; 64 x 64 x 16: 0.194, 0.212).
 constexpr int64_t kSerialSlabVox = int64_t(1) << 20;
 

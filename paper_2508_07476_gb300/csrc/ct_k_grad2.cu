@@ -657,10 +657,10 @@ int cta_width(int n0, int halo, double stage, const int* widths, int n) {
   return best;
 }
 
-// 16 warps per SM at every width, in CTAs that wait at their barriers
+// 16 warps per SM (15 at 96 and 160 columns), in CTAs that wait at their barriers
 // independently (512^3: 128 columns 0.62 ms, against 0.67 with two CTAs of 256).
-// The width that leaves the fewest idle columns: a 173-column row took two CTAs of 128,
-// now two of 96.
+// The width that covers the row with the least work: a 173-column row takes two CTAs
+// of 96, not two of 128.
 template <int RS>
 static cudaError_t launch_gxy_r(const uint16_t* vol, const Box& vb, const int dims[3], float* F, const Box& ab,
                                 const Taps& tx, const Taps& ty, int* zero, const Queue& st) {

@@ -129,11 +129,12 @@ struct Ha8 {
 // without branches and adds runs of equal bins to the CTA's shared histogram.
 // The depth's bin comes from an approximate square root; a depth within its
 // error of a bin edge is decided by the definition's arithmetic in a separate
-// rare loop, so that every count is the definition's. 
-// 512^3, FP32 HA, masked, 20 x 180 bins: 462 us with a thread's 8 voxels taken
-// where they lay, a square root each and 64-bit index divisions; 203 us now,
-// bound by the instructions of the bins (without them 89 us; the 402 MB that
-// it reads take 59 us at the copy rate).
+// rare loop, so that every count is the definition's.
+// 512^3, FP32 HA, masked, 20 x 180 bins: 203 us, bound by the instructions of the bins
+// (without them 89 us; the 402 MB that it reads take 59 us at the copy rate);
+// 462 us with a thread's 8 voxels taken where they lie, a square root each and
+// 64-bit index divisions.  Small fields gain less, the zeroing and flushing of the
+// bins being the same: 64^3 4.7 and 5.9 us, 128^3 9.3 and 12.1, 200^3 18.7 and 29.0.
 template <int TYPE, bool VEC>
 __global__ void __launch_bounds__(kProfThreads, kProfPerSm) k_transmural(const void* __restrict__ ha,
                                                                          const uint8_t* __restrict__ mask,

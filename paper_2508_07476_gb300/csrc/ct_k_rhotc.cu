@@ -1038,9 +1038,9 @@ struct TcLaunch {
     // x form: tensor maps when a group's rows are consecutive rows of one component
     // in the input box (its y extent is the output's) and in the output box.  A
     // component's last group may be ragged: the maps read its missing rows as zeros
-    // and clip them from the stores.  (Whole groups only, before: a haloed 384^3 chunk,
-    // whose 456^2 rows are not a multiple of 128, took a bulk copy per row, 843 us;
-    // 701 us now, 623 us at the copy rate for its bytes.)
+    // and clip them from the stores.  A haloed 384^3 chunk, whose 456^2 rows are not a
+    // multiple of 128: 701 us, with a bulk copy per row 843, 623 at the copy rate for
+    // its bytes.
     CUtensorMap tin, tout;
     std::memset(&tin, 0, sizeof tin);
     std::memset(&tout, 0, sizeof tout);

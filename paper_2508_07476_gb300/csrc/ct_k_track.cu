@@ -125,8 +125,8 @@ __device__ __forceinline__ int64_t nearest(const TrackDev& T, const float q[3]) 
   return ((int64_t)z * T.n[1] + y) * T.n[0] + x;
 }
 
-// 96 registers, 5 CTAs per SM (20.2 ms; bounded to 80 / 72 registers for 6 / 7
-// CTAs: 20.7 / 20.9 ms on the same board)
+// 96 registers, 5 CTAs per SM: bounded to 80 / 72 registers for 6 / 7 CTAs 3% slower
+// each, side by side
 constexpr int kTrackThreads = 128;
 __global__ void __launch_bounds__(kTrackThreads, 5) k_track(const float* __restrict__ vec, const float* __restrict__ fa,
                                                const uint8_t* __restrict__ mask, const float* __restrict__ seeds,

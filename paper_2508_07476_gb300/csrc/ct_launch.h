@@ -55,13 +55,11 @@ cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, size_t sme
 // of CTAs counted as they run side by side, the last one by the square root of
 // the share of an SM's CTAs it still holds (fewer CTAs run faster, but not in
 // proportion) and no less than kLoneCta (one waits for its own loads and
-// barriers).  seg: a multiple of unit.  Before, the walks were cut by powers of
-// two while the grid was below a fixed size and a segment above a fixed length,
-// so a 64^3 volume ran grad_z in 16 CTAs: its gradient x/y, z and rho z passes
-// 15.4, 16.4, 10.4 us, and 10.8, 8.3, 8.1 so; 173 x 141 x 118: gradient
-// 39.8 + 37.6 us, and 25.8 + 18.5.  The times are flat in the weights: kLoneCta
-// 0.25 .. 0.8 and warm x 0.6 .. 1.5 move none of the measured volumes by more
-// than 1%.
+// barriers).  seg: a multiple of unit.  64^3, gradient x/y, z and rho z passes:
+// 10.8, 8.3, 8.1 us, against 15.4, 16.4, 10.4 with cuts by powers of two above a
+// fixed length (grad_z then has 16 CTAs); 173 x 141 x 118, gradient: 25.8 + 18.5 and
+// 39.8 + 37.6.  The times are flat in the weights: kLoneCta 0.25 .. 0.8 and
+// warm x 0.6 .. 1.5 move none of the measured volumes by more than 1%.
 constexpr double kLoneCta = 0.5;
 inline int walk_segment(int64_t ctas, int n, int unit, double warm, int slots, int sms) {
   double best = 1e300;
@@ -199,13 +197,15 @@ cudaError_t launch_grad_xy_multi(const GxyItem* items, const MultiTable& T, int6
 uint3 grad_z_item(int rk, GzItem& it);
 cudaError_t launch_grad_z_multi(const GzItem* items, const MultiTable& T, int64_t blocks, const Taps& tz,
                                 const float scale[6], int rk, bool mixed, cudaStream_t st);
-// the fused x / y stencil at the CTA width `xt` (128 or 256; rho_xy_width picks it as the single launch does)
+// the fused x / y stencil at the CTA width `xt`: 128 or 256 (rho_xy_width; the single launch has
+// more widths to choose from)
 int rho_xy_width(int n0);
 uint3 rho_xy_item(int rk, int xt, RxyItem& it);
 cudaError_t launch_rho_xy_multi(const RxyItem* items, const MultiTable& T, int64_t blocks, const Taps& tx,
                                 const Taps& ty, int rk, int xt, cudaStream_t st);
-// the z stencil (axis 2), block_t outputs per thread block; the block shape
-// of an item: rho_stream_block (the single launch's), fixed per batch launch
+// the z stencil (axis 2) of k_rho_stream, block_t outputs per thread and block; the
+// block shape of an item: rho_stream_block, fixed per batch launch (the single
+// launch takes k_rho_z2 over even rows)
 uint3 rho_z_item(int rk, int block_t, dim3 block, RzItem& it);
 dim3 rho_stream_block(const Box& ob, int axis);
 cudaError_t launch_rho_z_multi(const RzItem* items, const MultiTable& T, int64_t blocks, dim3 block,
