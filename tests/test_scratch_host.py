@@ -22,7 +22,7 @@ def lib(tmp_path_factory):
     cxx = shutil.which("g++")
     if cxx is None:
         pytest.skip("no host compiler")
-    objs = [os.path.join(build.BUILD, f) for f in sorted(os.listdir(build.BUILD)) if f.endswith(".o")]
+    objs = [os.path.join(build.BUILD, f[:-3] + ".o") for f in sorted(os.listdir(build.CSRC)) if f.endswith(".cu")]
     out = str(tmp_path_factory.mktemp("double") / "libct_double.so")
     cuda = os.path.join(os.path.dirname(os.path.dirname(build.nvcc())), "include")
     subprocess.run([cxx, "-O1", "-std=c++17", "-shared", "-fPIC", "-Wl,-Bsymbolic", "-I", cuda,
